@@ -646,14 +646,31 @@ wlbm_status wlbm_init_temperature(wlbm_handle* h, const float* dT) {
   const Geom& g = h->g;
   h->scale = 1.f;
   if (h->storage == WLBM_STORE_BF16_DEV) {
-    // per-run scale: the largest |e_eq(T) - e_ref| of the start field and the walls
-    std::vector<float> host(size_t(g.nx) * g.ny);
-    wlbm_status st = h->cuda(cudaMemcpyAsync(host.data(), dT, host.size() * 4,
-                                             cudaMemcpyDeviceToHost, h->stream), "init");
+    // per-run scale: the largest |e_eq(T) - e_ref| of the start field and the walls.  e_eq
+    // grows with T > 0, so the field's smallest and largest value decide it.
+    const int64_t cells = int64_t(g.nx) * g.ny;
+    unsigned* range = reinterpret_cast<unsigned*>(h->d_red);
+    unsigned bits[2];
+    ++h->launches;
+    wlbm_status st = h->cuda(launch_range(dT, cells, range, h->stream), "init");
+    if (st == WLBM_OK)
+      st = h->cuda(cudaMemcpyAsync(bits, range, sizeof(bits), cudaMemcpyDeviceToHost, h->stream),
+                   "init");
     if (st == WLBM_OK) st = h->cuda(cudaStreamSynchronize(h->stream), "init");
     if (st != WLBM_OK) return st;
     double m = 0.0;
-    for (float v : host) m = std::max(m, std::fabs(h->delta_e(h->t_ref + double(v))));
+    float lo = 0.f, hi = 0.f;
+    const bool some = range_value(bits[0], &lo) && range_value(bits[1], &hi);
+    if (some && h->t_ref + double(lo) > 0.0) {
+      for (const float v : {lo, hi}) m = std::max(m, std::fabs(h->delta_e(h->t_ref + double(v))));
+    } else if (some) {   // no temperature: every cell counts
+      std::vector<float> host(static_cast<size_t>(cells));
+      st = h->cuda(cudaMemcpyAsync(host.data(), dT, host.size() * 4, cudaMemcpyDeviceToHost,
+                                   h->stream), "init");
+      if (st == WLBM_OK) st = h->cuda(cudaStreamSynchronize(h->stream), "init");
+      if (st != WLBM_OK) return st;
+      for (float v : host) m = std::max(m, std::fabs(h->delta_e(h->t_ref + double(v))));
+    }
     // values are stored relative to the local energy, so a fraction of the largest
     // deviation keeps them of order one
     for (int k = 0; k < 4; ++k)

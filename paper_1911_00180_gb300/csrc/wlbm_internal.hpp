@@ -439,6 +439,10 @@ cudaError_t launch_batch_persistent(int storage, int stages, const PersistArgs& 
                                     int grid, bool any_spec, cudaStream_t s);
 cudaError_t launch_walls(int storage, const WallArgs& a, cudaStream_t s);
 cudaError_t launch_periodic(int storage, const PeriodicArgs& a, cudaStream_t s);
+// Smallest and largest of n floats (NaN left out) as ordered bits into out[0], out[1]; the
+// value of such bits (false: none, every float was NaN).
+cudaError_t launch_range(const float* x, int64_t n, unsigned* out, cudaStream_t s);
+bool range_value(unsigned u, float* v);
 cudaError_t launch_init(int storage, const InitArgs& a, cudaStream_t s);
 cudaError_t launch_moments(int storage, const MomentArgs& a, cudaStream_t s);
 cudaError_t launch_reduce(int storage, const ReduceArgs& a, cudaStream_t s);
