@@ -285,6 +285,11 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
  *                          last boundary pass wrote (copies or wall values, not state).
  *                          Variant 3 never fuses the periodic mirrors: with
  *                          WLBM_OPT_FUSE_PERIODIC set it still runs the periodic pass.
+ *                          A grid whose planes fit the shared memory of one thread-block
+ *                          cluster (periodic or isothermal x sides; periodic, isothermal
+ *                          or diffuse y sides of specularity 0; no sources; the other
+ *                          options at their defaults) runs each chunk of steps as one
+ *                          launch, with the same results bit for bit.
  *   WLBM_OPT_GRAPH_STEPS   0 (default): launch every step's kernels directly; G > 0, a
  *                          multiple of 6: run chunks of G steps as one captured CUDA
  *                          graph (fewer launch gaps).  Replay needs a stream of its own:
@@ -333,7 +338,9 @@ wlbm_status wlbm_check(wlbm_handle* h);
  * (WLBM_OPT_GRAPH_STEPS = G) the timed launches are the steps t of each replayed chunk
  * with t % every == 0, recorded by event nodes of the graph; a graph's pairs are read
  * before it replays again (two chunks later: the host may wait for that replay to end).
- * Changing the stride drops the captured graphs.  WLBM_ERR_INVALID_ARG for every < 0.
+ * Changing the stride drops the captured graphs.  A launch that advances several steps
+ * counts once for each of its steps the stride selects, with that step's share of the
+ * launch's time.  WLBM_ERR_INVALID_ARG for every < 0.
  * wlbm_profile_read: synchronises the stream, returns the summed duration (ms) and count
  * of the timed step-kernel launches since the last read (then resets them), and the
  * number of kernels this handle has launched since it was created.  Any output may be

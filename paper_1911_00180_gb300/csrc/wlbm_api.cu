@@ -33,13 +33,20 @@ cudaError_t record_event(cudaEvent_t e, cudaStream_t s, bool node) {
   return node ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
 }
 
+// The steps an event pair around one launch stands for: `timed` of the launch's `of` steps
+// (a launch that advances several steps counts for each selected one its share).
+struct TimedSteps {
+  int timed = 1, of = 1;
+  double share(float ms) const { return double(ms) * timed / of; }
+};
+
 // One instantiated CUDA graph of a chunk of steps.  Captured while profiling, its timed
 // step-kernel launches record event pairs through event nodes; a replay overwrites them,
 // so they are read (waiting for that replay) before the graph replays again.
 struct TimedGraph {
   cudaGraphExec_t exec = nullptr;
   std::vector<cudaEvent_t> ev;   // (start, stop) pairs
-  int weight = 1;                // steps one pair times (a persistent launch: its steps)
+  std::vector<TimedSteps> steps; // what each pair times
   cudaEvent_t done = nullptr;    // recorded after every replay when there are pairs
   bool pending = false;          // replayed since the pairs were last read
 
@@ -59,11 +66,11 @@ struct TimedGraph {
     if (!pending) return cudaSuccess;
     pending = false;
     cudaError_t e = cudaEventSynchronize(done);
-    for (size_t k = 0; e == cudaSuccess && k + 1 < ev.size(); k += 2) {
+    for (size_t k = 0; e == cudaSuccess && k < steps.size(); ++k) {   // the pairs in use
       float t = 0.f;
-      e = cudaEventElapsedTime(&t, ev[k], ev[k + 1]);
-      *ms += t;
-      *n += weight;
+      e = cudaEventElapsedTime(&t, ev[2 * k], ev[2 * k + 1]);
+      *ms += steps[k].share(t);
+      *n += steps[k].timed;
     }
     return e;
   }
@@ -81,6 +88,7 @@ struct TimedGraph {
     if (done) cudaEventDestroy(done);
     exec = nullptr;
     ev.clear();
+    steps.clear();
     done = nullptr;
     pending = false;
   }
@@ -136,6 +144,7 @@ struct wlbm_handle {
   bool has_tmap_w = false;
   int bf16_wide = 0;          // variant 3, bfloat16: 1 = 256-column tiles (the default
                               // where the planes have a 32-bit-word tensor map)
+  ClusterArgs cluster{};      // many steps per launch of a small grid (nc = 0: not this grid)
   int graph_steps = 0;        // >0: replay chunks of this many steps as one CUDA graph
   int ring_stages = 0;        // variant 3 ring depth (0: by Q)
   int tile_loop = 0;          // variant 3: 1 = resident blocks loop over the tiles
@@ -188,6 +197,7 @@ struct wlbm_handle {
   int prof_every = 0;                 // time every prof_every-th step launch (0: none)
   int64_t prof_tick = 0;              // step launches seen while profiling
   std::vector<cudaEvent_t> prof_ev;   // pairs (start, stop)
+  std::vector<TimedSteps> prof_steps; // what each used pair times
   size_t prof_used = 0;
   double prof_graph_ms = 0.0;         // read from replayed graphs, not yet reported
   int64_t prof_graph_n = 0;
@@ -278,7 +288,13 @@ struct wlbm_handle {
       std::swap(e_cur, e_spare);
     }
   }
+  // The whole chunk in one launch: a small grid, the default step kernel, no sources.
+  bool cluster_on() const {
+    return cluster.nc > 0 && step_variant == 3 && ring_stages == 0 && tile_loop == 0 &&
+           n_src == 0 && !batch_owned && (!bf16() || bf16_wide);
+  }
   void build_wall_segments();
+  void plan_cluster();
 };
 
 // Ghost-cell segments handled by the wall kernel: non-periodic edges and the corners
@@ -332,6 +348,29 @@ void wlbm_handle::build_wall_segments() {
   a.mirror = mirror;
   a.scale = scale;
   a.inv_scale = inv_scale;
+}
+
+// Bands of the launch that advances many steps, for the walls it covers: periodic or isothermal
+// x sides, periodic, isothermal or diffuse y sides (specularity 0).
+void wlbm_handle::plan_cluster() {
+  cluster = ClusterArgs{};
+  auto row_ok = [&](int side) {
+    return bc_kind[side] == WLBM_BC_PERIODIC || bc_kind[side] == WLBM_BC_ISOTHERMAL ||
+           (bc_kind[side] == WLBM_BC_ADIABATIC_DIFFUSE && spec[side] == 0.f);
+  };
+  const bool x_ok = xper || (bc_kind[0] == WLBM_BC_ISOTHERMAL && bc_kind[1] == WLBM_BC_ISOTHERMAL);
+  // (one-column grids: the wall pass sums their diffuse ghost cells in another order)
+  if (g.nx < 2 || !x_ok || !row_ok(2) || !row_ok(3) || !has_tmap || (bf16() && !has_tmap_w)) return;
+  ClusterArgs a{};
+  a.planes = planes; a.plane = g.plane; a.pitch = g.pitch; a.nx = g.nx; a.ny = g.ny; a.q = g.q;
+  a.w = w_dev(); a.wfield = field_w ? wfield : nullptr; a.w0 = w0;
+  a.xper = xper; a.yper = yper; a.rho = rho_dev();
+  for (int s = 0; s < 2; ++s) a.row_kind[s] = bc_kind[2 + s];
+  for (int s = 0; s < 4; ++s)
+    a.iso[s] = bc_kind[s] == WLBM_BC_ISOTHERMAL ? float(delta_e(t_wall[s])) : 0.f;
+  a.y_first = bc_kind[2] == WLBM_BC_ADIABATIC_DIFFUSE ? -1 : 0;
+  a.y_last = bc_kind[3] == WLBM_BC_ADIABATIC_DIFFUSE ? g.ny : g.ny - 1;
+  if (cluster_plan(storage, &a)) cluster = a;
 }
 
 // Fill the periodic ghost cells (and their energies) from the current state, with plane
@@ -614,6 +653,7 @@ wlbm_status wlbm_create(const wlbm_grid* grid, const float* mfp_cells, double mf
   }
   if (e == cudaSuccess) e = prepare_step_kernels();
   if (e == cudaSuccess) e = configure_walls();
+  if (e == cudaSuccess) e = configure_step_cluster();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // host vectors die here
   if (e != cudaSuccess) {
     const std::string m = std::string("wlbm_create: ") + cudaGetErrorString(e);
@@ -621,6 +661,7 @@ wlbm_status wlbm_create(const wlbm_grid* grid, const float* mfp_cells, double mf
     return bad(WLBM_ERR_CUDA, m);
   }
   h->build_wall_segments();
+  h->plan_cluster();
   *out = h;
   return WLBM_OK;
 }
@@ -696,10 +737,53 @@ wlbm_status wlbm_init_temperature(wlbm_handle* h, const float* dT) {
 // every > 0: an event pair around every every-th step-kernel launch (counted across calls;
 // while capturing a graph, `cap` holds the graph's pairs and the steps t with t % every == 0
 // of the chunk are timed)
-static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every,
-                                 const std::vector<cudaEvent_t>* cap = nullptr) {
+static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every, TimedGraph* cap = nullptr) {
   size_t cap_used = 0;
   const Geom& g = h->g;
+  // An event pair for a launch of `of` steps, `timed` of them selected (none: null events).
+  auto timing = [&](int timed, int of, cudaEvent_t* e0, cudaEvent_t* e1) {
+    *e0 = *e1 = nullptr;
+    if (timed == 0) return WLBM_OK;
+    if (cap) {
+      *e0 = cap->ev[cap_used];
+      *e1 = cap->ev[cap_used + 1];
+      cap_used += 2;
+      cap->steps.push_back({timed, of});
+      return WLBM_OK;
+    }
+    while (h->prof_used + 2 > h->prof_ev.size()) {
+      cudaEvent_t ev;
+      const wlbm_status st = h->cuda(cudaEventCreate(&ev), "wlbm_step: profiling event");
+      if (st != WLBM_OK) return st;
+      h->prof_ev.push_back(ev);
+    }
+    *e0 = h->prof_ev[h->prof_used];
+    *e1 = h->prof_ev[h->prof_used + 1];
+    h->prof_used += 2;
+    h->prof_steps.push_back({timed, of});
+    return WLBM_OK;
+  };
+  auto selected = [&](int t) {
+    return every > 0 && (cap ? t % every == 0 : h->prof_tick++ % every == 0);
+  };
+  if (h->cluster_on()) {
+    int timed = 0;
+    for (int t = 0; t < count; ++t) timed += selected(t);
+    cudaEvent_t e0, e1;
+    wlbm_status st = timing(timed, count, &e0, &e1);
+    if (st == WLBM_OK && e0)
+      st = h->cuda(record_event(e0, h->stream, cap != nullptr), "wlbm_step: profiling");
+    if (st != WLBM_OK) return st;
+    ClusterArgs a = h->cluster;
+    a.codes = h->d_codes; a.order = h->d_order; a.steps = count;
+    a.e = h->e[h->e_cur]; a.e_ref = h->ref_plane();
+    a.scale = h->scale; a.inv_scale = h->inv_scale;
+    st = h->cuda(launch_step_cluster(h->storage, a, h->stream), "wlbm_step: steps");
+    ++h->launches;
+    if (st == WLBM_OK && e1)
+      st = h->cuda(record_event(e1, h->stream, cap != nullptr), "wlbm_step: profiling");
+    return st;
+  }
   const bool any_wall = h->walls.nseg > 0;
   // both axes periodic: the step kernel mirrors the edges itself (grids of 2+ cells)
   // (variant 3 has no mirror stores: there the separate periodic pass runs)
@@ -754,28 +838,11 @@ static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every,
     sa.order = h->d_order + size_t(t) * (g.q + 17);
     int tx_unused = 0, ty_unused = 0;
     tma_cover(h->bc_kind, g.nx, g.ny, &sa, &tx_unused, &ty_unused);
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (every > 0 && (cap ? t % every == 0 : h->prof_tick++ % every == 0)) {
-      if (cap) {
-        e0 = (*cap)[cap_used];
-        e1 = (*cap)[cap_used + 1];
-        cap_used += 2;
-      } else {
-        if (h->prof_used + 2 > h->prof_ev.size()) {
-          for (int k = 0; k < 2; ++k) {
-            cudaEvent_t ev;
-            st = h->cuda(cudaEventCreate(&ev), "wlbm_step: profiling event");
-            if (st != WLBM_OK) return st;
-            h->prof_ev.push_back(ev);
-          }
-        }
-        e0 = h->prof_ev[h->prof_used];
-        e1 = h->prof_ev[h->prof_used + 1];
-        h->prof_used += 2;
-      }
+    cudaEvent_t e0, e1;
+    st = timing(selected(t) ? 1 : 0, 1, &e0, &e1);
+    if (st == WLBM_OK && e0)
       st = h->cuda(record_event(e0, h->stream, cap != nullptr), "wlbm_step: profiling");
-      if (st != WLBM_OK) return st;
-    }
+    if (st != WLBM_OK) return st;
     st = h->cuda(launch_step(h->storage, sa, h->stream), "wlbm_step: step");
     if (st != WLBM_OK) return st;
     ++h->launches;
@@ -812,7 +879,7 @@ static wlbm_status run_graph(wlbm_handle* h) {
       tg.destroy();
       return st;
     }
-    const wlbm_status est = enqueue_steps(h, G, every, &tg.ev);
+    const wlbm_status est = enqueue_steps(h, G, every, &tg);
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(h->stream, &graph);
     if (est != WLBM_OK) {
@@ -969,16 +1036,19 @@ wlbm_status wlbm_profile_read(wlbm_handle* h, double* step_ms, int64_t* step_lau
       if (st != WLBM_OK) return st;
     }
   double total = h->prof_graph_ms;
+  int64_t timed = h->prof_graph_n;
   for (size_t k = 0; k + 1 < h->prof_used; k += 2) {
     float ms = 0.f;
     st = h->cuda(cudaEventElapsedTime(&ms, h->prof_ev[k], h->prof_ev[k + 1]), "wlbm_profile_read");
     if (st != WLBM_OK) return st;
-    total += ms;
+    total += h->prof_steps[k / 2].share(ms);
+    timed += h->prof_steps[k / 2].timed;
   }
   if (step_ms) *step_ms = total;
-  if (step_launches) *step_launches = h->prof_graph_n + int64_t(h->prof_used / 2);
+  if (step_launches) *step_launches = timed;
   if (all_launches) *all_launches = h->launches;
   h->prof_used = 0;
+  h->prof_steps.clear();
   h->prof_graph_ms = 0.0;
   h->prof_graph_n = 0;
   return WLBM_OK;
@@ -2083,8 +2153,7 @@ wlbm_status wlbm_batch_set_option(wlbm_batch* b, int32_t key, int64_t value) {
 }  // extern "C"
 
 // Kernels of `count` steps for the whole batch, instance records already on the device.
-static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every,
-                                 const std::vector<cudaEvent_t>* cap = nullptr) {
+static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every, TimedGraph* cap = nullptr) {
   size_t cap_used = 0;
   const int n = int(b->h.size());
   wlbm_status st = WLBM_OK;
@@ -2126,8 +2195,9 @@ static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every,
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (every > 0) {
       if (cap) {
-        e0 = (*cap)[0];
-        e1 = (*cap)[1];
+        e0 = cap->ev[0];
+        e1 = cap->ev[1];
+        cap->steps.push_back({count, count});
       } else {
         if (b->prof_used + 2 > b->prof_ev.size()) {
           for (int j = 0; j < 2; ++j) {
@@ -2178,9 +2248,10 @@ static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every,
     if (every > 0 && (cap ? t % every == 0 : b->prof_tick++ % every == 0)) {
       cudaEvent_t e0 = nullptr;
       if (cap) {
-        e0 = (*cap)[cap_used];
-        e1 = (*cap)[cap_used + 1];
+        e0 = cap->ev[cap_used];
+        e1 = cap->ev[cap_used + 1];
         cap_used += 2;
+        cap->steps.push_back({});
       } else {
         if (b->prof_used + 2 > b->prof_ev.size()) {
           for (int j = 0; j < 2; ++j) {
@@ -2285,7 +2356,6 @@ wlbm_status wlbm_batch_step(wlbm_batch* b, int64_t n) {
         const int every = b->prof_every;
         // a persistent chunk is one launch: one timed pair covering its ch steps
         const int pairs = every > 0 ? (b->persistent ? 1 : (ch + every - 1) / every) : 0;
-        fresh.weight = b->persistent ? ch : 1;
         st = b->cuda(fresh.make_events(pairs), "wlbm_batch_step: graph events");
         const int64_t l0 = b->launches;
         if (st == WLBM_OK)
@@ -2295,7 +2365,7 @@ wlbm_status wlbm_batch_step(wlbm_batch* b, int64_t n) {
           fresh.destroy();
           return st;
         }
-        const wlbm_status est = batch_enqueue(b, ch, every, &fresh.ev);
+        const wlbm_status est = batch_enqueue(b, ch, every, &fresh);
         cudaGraph_t gr = nullptr;
         const cudaError_t ce = cudaStreamEndCapture(b->stream, &gr);
         if (est == WLBM_OK) st = b->cuda(ce, "wlbm_batch_step: capture");

@@ -90,6 +90,28 @@ struct StepArgs {
   const void* tmap_w;
 };
 
+// Many steps of a small grid in one launch (k_step_cluster.cu).
+struct ClusterArgs {
+  void* planes;           // [2][q][plane] current planes, read and written
+  int64_t plane;
+  int pitch, nx, ny, q;
+  const uint8_t* codes;   // [steps][q]
+  const uint16_t* order;  // [steps][q + 17] kind-sorted directions
+  int steps;
+  const float* w;
+  float* e;               // local energy and (bfloat16) reference energy, read and written
+  float* e_ref;
+  const float* wfield;
+  float w0, scale, inv_scale;
+  int xper, yper;
+  int row_kind[2];        // wall kinds of y-, y+ (WLBM_BC_ISOTHERMAL or _ADIABATIC_DIFFUSE)
+  float iso[4];           // e_eq(T_w) - e_ref of isothermal walls
+  const float* rho;       // [8][q] re-emission fractions
+  int y_first, y_last;    // computed cell rows (diffuse ghost rows included)
+  // set by cluster_plan: blocks, whether a block takes rows or columns, how many, threads
+  int nc, split_rows, per, threads;
+};
+
 // Stable sort of one step's directions by kind = hop | paused << 3 (16 kinds): writes the
 // sorted direction indices to out[0..q) and the start of every kind to out[q..q+17).
 inline void sort_by_kind(const uint8_t* codes, int q, uint16_t* out) {
@@ -423,6 +445,11 @@ cudaError_t configure_adj_tma();
 cudaError_t launch_adj_tma(const AdjArgs& a, const void* lam_map, const void* lam_map14,
                            const void* tape_map, int tape_z0, const uint16_t* order,
                            int* status, cudaStream_t s);
+// Small grids: attributes, the bands of the cluster that holds the state (false when it does
+// not fit; fields up to y_last must be set but codes, order and steps) and the launch.
+cudaError_t configure_step_cluster();
+bool cluster_plan(int storage, ClusterArgs* a);
+cudaError_t launch_step_cluster(int storage, const ClusterArgs& a, cudaStream_t s);
 // Batched launches (one launch per step for all instances of a batch).
 int step_tile_width(int storage, int variant);
 cudaError_t launch_step_batch(int storage, int variant, const BatchInst* insts, int n,
