@@ -398,9 +398,8 @@ wlbm_status wlbm_autotune(wlbm_handle* h, int32_t trial_steps, int32_t* variant,
  * every instance has a tensor map), WLBM_OPT_GRAPH_STEPS, WLBM_OPT_FUSE_PERIODIC, and
  * WLBM_OPT_BF16_WIDE (bfloat16 per-step launches of variant 3 in 256-column tiles; default
  * 1 when every instance has a word tensor map; the persistent kernel keeps 128 columns).
- * Instances with a periodic axis whose edges the step kernel does not mirror get their own
- * periodic pass each step; graph replay then keeps one captured graph per starting
- * energy-plane phase of those instances (at most three).  Options of batches only:
+ * Instances with a periodic axis whose edges the step kernel does not mirror share one
+ * periodic pass each step.  Options of batches only:
  *   WLBM_OPT_PERSISTENT    0 (default): one wall launch and one step launch per step; 1:
  *                          one persistent launch per chunk of steps (64, or the
  *                          WLBM_OPT_GRAPH_STEPS of a replayed graph) on a fixed grid of

@@ -1780,16 +1780,12 @@ struct wlbm_batch {
   std::vector<size_t> code_off, order_off;   // order_off in uint16 elements
   size_t code_bytes = 0, order_elems = 0;
   int total_tiles = 0, total_wall_blocks = 0;
-  std::vector<int> per;             // instances whose periodic edges need their own launch
-  // Captured chunks, keyed by the energy-plane phases of the instances in `per` (their
-  // periodic launches bake plane pointers; the batched kernels read phases at run time).
-  // Two per key (replay parity), as for a single grid.
-  struct Graph {
-    std::vector<int> key;
-    int parity = 0;
-    TimedGraph tg;
-  };
-  std::vector<Graph> graphs;
+  std::vector<int> per;             // instances whose periodic edges need the separate pass
+  int2* d_per = nullptr;            // {instance, its first block column} of every block column
+  int per_cap = 0, per_blocks = 0, per_q = 0;   // of that pass; the largest Q among them
+  // A captured chunk (the batched kernels read planes and phases at run time), two for the
+  // replay parities, as for a single grid.
+  TimedGraph graphs[2];
   int graph_parity = 0;
   int64_t graph_replays = 0;
   int64_t graph_launches = 0, launches = 0;
@@ -1822,16 +1818,10 @@ struct wlbm_batch {
     return p;
   }
   void drop_graph() {
-    for (Graph& gr : graphs) {
-      gr.tg.harvest(&prof_graph_ms, &prof_graph_n);
-      gr.tg.destroy();
+    for (TimedGraph& tg : graphs) {
+      tg.harvest(&prof_graph_ms, &prof_graph_n);
+      tg.destroy();
     }
-    graphs.clear();
-  }
-  std::vector<int> phase_key() const {
-    std::vector<int> key;
-    for (int k : per) key.push_back(h[k]->e_cur);
-    return key;
   }
   void release() {
     drop_graph();
@@ -1873,10 +1863,29 @@ struct wlbm_batch {
   bool wraps(const wlbm_handle* x) const {
     return fuse_periodic && variant != 3 && x->xper && x->yper && x->g.nx >= 2 && x->g.ny >= 2;
   }
-  void classify() {
+  // Instances of the periodic pass and its block table (false: it could not be uploaded).
+  bool classify() {
     per.clear();
-    for (size_t k = 0; k < h.size(); ++k)
-      if ((h[k]->xper || h[k]->yper) && !wraps(h[k])) per.push_back(int(k));
+    std::vector<int2> blocks;
+    per_q = 0;
+    for (size_t k = 0; k < h.size(); ++k) {
+      const wlbm_handle* x = h[k];
+      if (!(x->xper || x->yper) || wraps(x)) continue;
+      per.push_back(int(k));
+      per_q = std::max(per_q, x->g.q);
+      const int first = int(blocks.size());
+      blocks.insert(blocks.end(), size_t(periodic_blocks(x->g.nx, x->g.ny, x->xper, x->yper)),
+                    make_int2(int(k), first));
+    }
+    per_blocks = int(blocks.size());
+    if (per_blocks == 0) return true;
+    if (per_blocks > per_cap) {
+      d_per = static_cast<int2*>(dev_alloc(blocks.size() * sizeof(int2)));
+      per_cap = d_per ? per_blocks : 0;
+    }
+    return d_per && (!stream || cudaStreamSynchronize(stream) == cudaSuccess) &&
+           cudaMemcpy(d_per, blocks.data(), blocks.size() * sizeof(int2),
+                      cudaMemcpyHostToDevice) == cudaSuccess;
   }
   // Block and warp offsets of every instance in the batched grids.
   void layout() {
@@ -1971,7 +1980,6 @@ wlbm_status wlbm_batch_create(int32_t n, const wlbm_grid* grids, const float* co
       return bad(WLBM_ERR_INVALID_ARG, "wlbm_batch_create: all instances need one storage type");
   }
   b->storage = grids[0].storage;
-  b->classify();
   b->code_off.resize(n);
   b->order_off.resize(n);
   b->all_tmap = true;
@@ -2027,16 +2035,13 @@ wlbm_status wlbm_batch_create(int32_t n, const wlbm_grid* grids, const float* co
     return bad(WLBM_ERR_CUDA, std::string("wlbm_batch_create: ") + cudaGetErrorString(e));
   }
   std::memset(b->h_inst, 0, sizeof(BatchInst) * n);
-  if (b->all_tmap) {
-    b->variant = 3;
-    b->classify();
-  }
+  if (b->all_tmap) b->variant = 3;
   b->wide = b->all_tmap_w ? 1 : 0;
   std::memset(b->h_walls, 0, sizeof(BatchWalls) * n);
   b->layout();
-  if (!b->tables_ok) {
+  if (!b->classify() || !b->tables_ok) {
     cudaGetLastError();
-    return bad(WLBM_ERR_CUDA, "wlbm_batch_create: upload of the tile tables failed");
+    return bad(WLBM_ERR_CUDA, "wlbm_batch_create: upload of the block tables failed");
   }
   *out = b;
   return WLBM_OK;
@@ -2095,11 +2100,10 @@ wlbm_status wlbm_batch_set_option(wlbm_batch* b, int32_t key, int64_t value) {
                      "wlbm_batch_set_option: the persistent kernel runs variant 3");
     b->variant = int(value);
     b->layout();
-    b->classify();
     b->drop_graph();
-    if (!b->tables_ok) {
+    if (!b->classify() || !b->tables_ok) {
       cudaGetLastError();
-      return b->fail(WLBM_ERR_CUDA, "wlbm_batch_set_option: upload of the tile tables failed");
+      return b->fail(WLBM_ERR_CUDA, "wlbm_batch_set_option: upload of the block tables failed");
     }
     return WLBM_OK;
   }
@@ -2135,8 +2139,11 @@ wlbm_status wlbm_batch_set_option(wlbm_batch* b, int32_t key, int64_t value) {
   }
   if (key == WLBM_OPT_FUSE_PERIODIC && (value == 0 || value == 1)) {
     b->fuse_periodic = int(value);
-    b->classify();
     b->drop_graph();
+    if (!b->classify()) {
+      cudaGetLastError();
+      return b->fail(WLBM_ERR_CUDA, "wlbm_batch_set_option: upload of the block tables failed");
+    }
     return WLBM_OK;
   }
   if (key == WLBM_OPT_BF16_WIDE && (value == 0 || value == 1)) {
@@ -2229,18 +2236,9 @@ static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every, TimedGraph
                    "wlbm_batch_step: walls");
       ++b->launches;
     }
-    for (int k : b->per) {
-      if (st != WLBM_OK) break;
-      wlbm_handle* x = b->h[k];
-      const Geom& g = x->g;
-      const BatchInst& I = b->h_inst[k];
-      const int cur = (I.phase + t) % I.n_e;
-      PeriodicArgs pa{};
-      pa.planes = x->planes; pa.plane = g.plane; pa.pitch = g.pitch; pa.nx = g.nx; pa.ny = g.ny;
-      pa.q = g.q; pa.codes = b->d_codes + b->code_off[k] + size_t(t) * g.q;
-      pa.e_cur = I.e[cur]; pa.e_ref = I.n_e == 3 ? I.e[(cur + 2) % 3] : nullptr;
-      pa.xper = x->xper; pa.yper = x->yper;
-      st = b->cuda(launch_periodic(b->storage, pa, b->stream), "wlbm_batch_step: periodic");
+    if (st == WLBM_OK && b->per_blocks > 0) {
+      st = b->cuda(launch_periodic_batch(b->storage, b->d_inst, b->d_per, b->per_blocks, b->per_q, t,
+                                         b->stream), "wlbm_batch_step: periodic");
       ++b->launches;
     }
     if (st != WLBM_OK) break;
@@ -2344,14 +2342,9 @@ wlbm_status wlbm_batch_step(wlbm_batch* b, int64_t n) {
     if (st == WLBM_OK) st = b->cuda(cudaEventRecord(b->ev, b->stream), "wlbm_batch_step");
     if (st != WLBM_OK) return st;
     if (graphs && ch == b->graph_steps) {
-      const std::vector<int> key = b->phase_key();
-      const int parity = b->graph_parity;
+      TimedGraph* tg = &b->graphs[b->graph_parity];
       b->graph_parity ^= 1;
-      TimedGraph* tg = nullptr;
-      for (wlbm_batch::Graph& gr : b->graphs)
-        if (gr.key == key && gr.parity == parity) tg = &gr.tg;
-      if (!tg) {
-        if (b->graphs.size() >= 6) b->drop_graph();
+      if (!tg->exec) {
         TimedGraph fresh;
         const int every = b->prof_every;
         // a persistent chunk is one launch: one timed pair covering its ch steps
@@ -2377,8 +2370,7 @@ wlbm_status wlbm_batch_step(wlbm_batch* b, int64_t n) {
           fresh.destroy();
           return st;
         }
-        b->graphs.push_back({key, parity, fresh});
-        tg = &b->graphs.back().tg;
+        *tg = fresh;
         b->graph_launches = b->launches - l0;
         b->launches = l0;
       } else {
@@ -2430,8 +2422,8 @@ wlbm_status wlbm_batch_profile_read(wlbm_batch* b, double* step_ms, int64_t* ste
   if (!b) return WLBM_ERR_INVALID_ARG;
   wlbm_status st = b->cuda(cudaStreamSynchronize(b->stream), "wlbm_batch_profile_read");
   if (st != WLBM_OK) return st;
-  for (wlbm_batch::Graph& gr : b->graphs) {
-    st = b->cuda(gr.tg.harvest(&b->prof_graph_ms, &b->prof_graph_n), "profile_read");
+  for (TimedGraph& tg : b->graphs) {
+    st = b->cuda(tg.harvest(&b->prof_graph_ms, &b->prof_graph_n), "profile_read");
     if (st != WLBM_OK) return st;
   }
   double total = b->prof_graph_ms;

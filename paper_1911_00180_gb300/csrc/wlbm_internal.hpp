@@ -466,6 +466,12 @@ cudaError_t launch_batch_persistent(int storage, int stages, const PersistArgs& 
                                     int grid, bool any_spec, cudaStream_t s);
 cudaError_t launch_walls(int storage, const WallArgs& a, cudaStream_t s);
 cudaError_t launch_periodic(int storage, const PeriodicArgs& a, cudaStream_t s);
+// Blocks per plane of a grid's periodic pass, and the pass of step t of every instance of a batch
+// that needs one: total_blocks block columns, blocks[b] = {instance, its first column}; max_q
+// the largest Q among them.
+int periodic_blocks(int nx, int ny, int xper, int yper);
+cudaError_t launch_periodic_batch(int storage, const BatchInst* insts, const int2* blocks,
+                                  int total_blocks, int max_q, int t, cudaStream_t s);
 // Smallest and largest of n floats (NaN left out) as ordered bits into out[0], out[1]; the
 // value of such bits (false: none, every float was NaN).
 cudaError_t launch_range(const float* x, int64_t n, unsigned* out, cudaStream_t s);
