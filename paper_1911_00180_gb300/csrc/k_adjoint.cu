@@ -358,6 +358,18 @@ __global__ void k_adj_seed(const AdjArgs a, const float* dJ_dT, const float* dJ_
 __global__ void k_adj_final(const AdjArgs a, const float* dwc, float* dJ_dmfp,
                             const float* lam0, const float* s0, const float* dT0,
                             float* dJ_ddT0, double t_ref, double theta) {
+  // weights as float64, and their sum, once a block: the float64 pipe bounds this kernel
+  __shared__ double sw[kMaxQ];
+  __shared__ double swsum;
+  for (int i = int(threadIdx.x); i < a.q; i += int(blockDim.x)) sw[i] = double(a.w[i]);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int i = 0; i < a.q; ++i) sum += sw[i];
+    swsum = sum;
+  }
+  __syncthreads();
+  const double wsum = swsum;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nx * a.ny) return;
   const int y = t / a.nx, x = t - y * a.nx;
@@ -372,11 +384,9 @@ __global__ void k_adj_final(const AdjArgs a, const float* dwc, float* dJ_dmfp,
         if (jx > 0 && fx[jx] == x) continue;
         const int64_t off = int64_t(fy[jy] + 2) * a.pitch + (fx[jx] + kX0);
         // l^0_i = lh_i + s, so sum_i w_i l^0_i = sum_i w_i lh_i + s sum_i w_i
-        double s = 0.0, wsum = 0.0;
-        for (int i = 0; i < a.q; ++i) {
-          s += double(a.w[i]) * lam0[int64_t(i) * a.plane + off];
-          wsum += double(a.w[i]);
-        }
+        double s = 0.0;
+#pragma unroll 8
+        for (int i = 0; i < a.q; ++i) s += sw[i] * lam0[int64_t(i) * a.plane + off];
         acc += s + wsum * double(s0[off]);
       }
     }

@@ -206,25 +206,58 @@ __global__ void __launch_bounds__(256) k_range(const float* x, int64_t n, unsign
   }
 }
 
+// float(double(w) * de), the product rounded to float64 and then to float32, mostly without
+// the float64 pipe (2 operations a cycle and SM): de = hi + lo, and ph + s with ph = w hi
+// rounded and s its exact remainder + w lo is within |ph| 2^-44 of the float64 product
+// (de - hi - lo <= 2^-48 |de|, s rounds to 2^-47 |ph|, the product itself to 2^-53).  Rounding
+// is monotonic, so where both ends of that interval round to the same float32 it is the
+// result; else (one value in some 2^19, and products too small to split) float64 decides.
+struct SplitDouble {
+  double d;
+  float hi, lo;
+  bool small;   // w hi 2^-44 could leave the normal float32 range
+};
+__device__ __forceinline__ SplitDouble split_double(double d) {
+  const float hi = float(d);
+  return {d, hi, float(d - double(hi)), !(fabsf(hi) > 1e-18f && fabsf(hi) < 1e30f)};
+}
+// a call, so that the float64 instructions are not issued under a false predicate
+__device__ __noinline__ float product64(float w, double d) { return float(double(w) * d); }
+__device__ __forceinline__ float round_product(float w, const SplitDouble& x) {
+  const float ph = __fmul_rn(w, x.hi);
+  const float s = fmaf(w, x.lo, fmaf(w, x.hi, -ph));
+  const float tol = fabsf(ph) * 0x1p-44f;
+  const float r0 = __fadd_rn(ph, __fsub_rn(s, tol)), r1 = __fadd_rn(ph, __fadd_rn(s, tol));
+  return r0 == r1 && !x.small ? r0 : product64(w, x.d);
+}
+
+// Bound by the state's write and a cell's expm1 once the products leave the float64 pipe, which
+// took three of its operations a value (bfloat16: six): 4096 x 256 x Q128 825 -> 160 us
+// (bfloat16 1581 -> 176).
 template <typename T>
-__global__ void k_init(const InitArgs a) {
+__global__ void __launch_bounds__(256) k_init(const InitArgs a) {
+  __shared__ float sw[kMaxQ];
+  for (int i = int(threadIdx.x); i < a.q; i += 256) sw[i] = a.w[i];
+  __syncthreads();
   const int fw = a.nx + 2, fh = a.ny + 2;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= fw * fh) return;
   const int fy = t / fw, fx = t - fy * fw;            // framed coordinates
   const int x = min(max(fx - 1, 0), a.nx - 1), y = min(max(fy - 1, 0), a.ny - 1);
   const double temp = a.t_ref + double(a.dT[int64_t(y) * a.nx + x]);
-  const double de = 1.0 / expm1(a.theta / temp) - a.e_ref;
+  const SplitDouble de = split_double(1.0 / expm1(a.theta / temp) - a.e_ref);
   const int64_t off = int64_t(fy + 1) * a.pitch + (kGhostCol + fx);
   T* planes = static_cast<T*>(a.planes);
   if (a.e_refp) {   // reference energy = the equilibrium energy of this cell
     float e0 = 0.f;
-    for (int i = 0; i < a.q; ++i) e0 += float(double(a.w[i]) * de);
+#pragma unroll 8
+    for (int i = 0; i < a.q; ++i) e0 += round_product(sw[i], de);
     a.e_refp[off] = e0;
   }
   float e = 0.f;
+#pragma unroll 8
   for (int i = 0; i < a.q; ++i)
-    e += dev_store(planes + int64_t(i) * a.plane + off, float(double(a.w[i]) * de), a.w[i],
+    e += dev_store(planes + int64_t(i) * a.plane + off, round_product(sw[i], de), sw[i],
                    a.e_refp, off, a.scale, a.inv_scale);
   a.e_cur[off] = e;
 }
