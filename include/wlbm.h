@@ -308,6 +308,9 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
  *                          single grids take these 128-column forms with
  *                          WLBM_OPT_BF16_WIDE = 0 or the tile loop; batches with
  *                          WLBM_OPT_BF16_WIDE = 0 take the cell-tile form with 8 stages.
+ *                          With 0 single grids of about one tile per SM or fewer take a
+ *                          kernel of one cell per thread instead.  Same results bit for
+ *                          bit.
  *   WLBM_OPT_TILE_LOOP     variant 3: 0 (default) one block per 128 x 14 tile; 1 a grid of
  *                          resident blocks that take the tiles in turn (no partial last
  *                          wave; bfloat16 runs three such blocks per SM where the ring

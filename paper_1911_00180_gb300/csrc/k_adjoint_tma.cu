@@ -322,6 +322,7 @@ cudaError_t launch_adj_tma(const AdjArgs& a, const void* lam_map, const void* la
                            int* status, cudaStream_t s) {
   const dim3 block(32, kAW + 1);
   const dim3 grid((kX0 + a.nx - kAC0) / kATW + 1, (a.ny + 2 + kARows - 1) / kARows);
+  if (adj_direct_ok(a, int(grid.x * grid.y))) return launch_adj_direct(a, order, s);
   k_adj_tma<<<grid, block, adj_tma_bytes(a.q), s>>>(
       a, *static_cast<const CUtensorMap*>(lam_map), *static_cast<const CUtensorMap*>(lam_map14),
       *static_cast<const CUtensorMap*>(tape_map), tape_z0, order, status);

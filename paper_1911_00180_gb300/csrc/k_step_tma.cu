@@ -379,6 +379,7 @@ int step_tma_loop_blocks(int storage, int stages, bool field_w, int q) {
 }
 
 cudaError_t launch_step_tma(int storage, const StepArgs& a, cudaStream_t s) {
+  if (step_is_direct(storage, a)) return launch_step_direct(storage, a, s);
   const CUtensorMap& tm = *static_cast<const CUtensorMap*>(a.tmap);
   const int st = single_stages(storage, a.ring_stages, a.q);
   if (storage == WLBM_STORE_BF16_DEV) {

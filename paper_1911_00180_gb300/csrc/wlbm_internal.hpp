@@ -404,6 +404,9 @@ cudaError_t configure_walls();        // the same for the single-grid wall pass
 // `out`, 128 bytes, 64-byte aligned; false with a reason when it cannot be made).
 cudaError_t configure_step_tma();
 cudaError_t launch_step_tma(int storage, const StepArgs& a, cudaStream_t s);
+// Whether launch_step_tma takes the direct-load kernel (k_step_direct.cu).
+bool step_is_direct(int storage, const StepArgs& a);
+cudaError_t launch_step_direct(int storage, const StepArgs& a, cudaStream_t s);
 // Ring depths compiled for single grids (0 picks by Q) and the blocks of the tile-looping
 // grid for this storage, depth, W kind and Q (resident blocks per SM x SMs; 0 on error).
 bool step_tma_stages_ok(int storage, int stages);
@@ -442,6 +445,9 @@ constexpr int kAdjTmaBoxRows = 15;
 constexpr int kAdjTmaRows = 14;
 constexpr int kAdjTmaCols = 128;
 cudaError_t configure_adj_tma();
+// Direct-load reverse step of a grid whose TMA form would be `tiles` blocks.
+bool adj_direct_ok(const AdjArgs& a, int tiles);
+cudaError_t launch_adj_direct(const AdjArgs& a, const uint16_t* order, cudaStream_t s);
 cudaError_t launch_adj_tma(const AdjArgs& a, const void* lam_map, const void* lam_map14,
                            const void* tape_map, int tape_z0, const uint16_t* order,
                            int* status, cudaStream_t s);
