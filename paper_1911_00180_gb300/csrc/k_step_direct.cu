@@ -145,7 +145,9 @@ constexpr int kAdjU = 4;
 __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_direct(const AdjArgs a,
                                                                const uint16_t* order) {
   __shared__ float sS[kAdjTile];
-  __shared__ float hwall[4];   // isothermal harvest of this block per wall
+  // isothermal harvest of the block's rows at the x walls, added as k_adj_tma's warps of two
+  // rows mostly do: each warp's first row, then each warp's second
+  __shared__ float hrow[2][kAdjTmaRows];
   extern __shared__ __align__(16) unsigned char smem[];
   DirectAdj* table = reinterpret_cast<DirectAdj*>(smem);
   const int tid = int(threadIdx.x), lane = tid & 31, ty = tid >> 5;
@@ -158,7 +160,8 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_direct(const AdjArgs a,
     table[j] = {int(k * a.plane), cy * a.pitch + cx, a.w[k], int16_t(cy * kSW + cx),
                 int16_t(code & 8)};
   }
-  if (tid < 4) hwall[tid] = 0.f;
+  if (tid < 2 * kAdjTmaRows) hrow[tid / kAdjTmaRows][tid % kAdjTmaRows] = 0.f;
+  step_waits();
 #pragma unroll
   for (int h = 0; h < (kAdjTile + kAdjThreads - 1) / kAdjThreads; ++h) {
     const int idx = tid + h * kAdjThreads;
@@ -216,11 +219,16 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_direct(const AdjArgs a,
     }
     a.s_out[cell] = W * sigma;
     a.gw[cell] += fmaf(sigma - a0, ed, -pd);
-    if (harvest) atomicAdd(&hwall[iso], hs);
+    if (harvest) hrow[col == kGhostCol ? 0 : 1][ty] = hs;
   }
   // one global atomic per wall and block
-  if (__syncthreads_or(harvest) && tid < 4 && hwall[tid] != 0.f)
-    atomicAdd(a.gtw + tid, double(hwall[tid]));
+  if (__syncthreads_or(harvest) && tid < 2) {
+    float sum = 0.f;
+    for (int r = 0; r < kAdjTmaRows; r += 2) sum += hrow[tid][r];
+    for (int r = 1; r < kAdjTmaRows; r += 2) sum += hrow[tid][r];
+    const int iso = a.iso_side[tid];
+    if (iso >= 0 && sum != 0.f) atomicAdd(a.gtw + iso, double(sum));
+  }
 }
 
 template <typename T>
