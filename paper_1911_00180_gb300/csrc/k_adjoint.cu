@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(32 * kAdjRows) k_adj_step(const AdjArgs a) {
 // Transpose of the periodic x link (all frame rows), then of the y link.
 __global__ void k_periodic_T_x(float* planes, int64_t plane, int pitch, int nx, int ny,
                                int nplanes) {
+  step_waits();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (ny + 2) * nplanes) return;
   const int p = t / (ny + 2), r = 1 + (t - p * (ny + 2));
@@ -193,6 +194,7 @@ __global__ void k_periodic_T_x(float* planes, int64_t plane, int pitch, int nx, 
 
 __global__ void k_periodic_T_y(float* planes, int64_t plane, int pitch, int nx, int ny,
                                int nplanes, int xper) {
+  step_waits();
   const int ncol = xper ? nx : nx + 2, c0 = xper ? kX0 : kGhostCol;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ncol * nplanes) return;
@@ -253,6 +255,7 @@ __device__ __forceinline__ float walls_T_cell(const WallArgs& wa, const WallSeg&
 __global__ void __launch_bounds__(32 * kWallWarpsT) k_walls_T(const WallArgs wa, float* lam,
                                                                double* gtw) {
   __shared__ float part_s[kWallWarpsT * 32 * 4];
+  step_waits();
   int c = 0;
   const int s = wall_chunk_segment(wa.nseg, wa.seg, int(blockIdx.x), &c);
   if (s >= wa.nseg) return;
@@ -410,18 +413,18 @@ cudaError_t launch_adj_step(const AdjArgs& a, cudaStream_t s) {
 cudaError_t launch_periodic_T(float* planes, int64_t plane, int pitch, int nx, int ny,
                               int nplanes, int xper, int yper, cudaStream_t s) {
   if (xper)
-    k_periodic_T_x<<<nblk(int64_t(ny + 2) * nplanes, 256), 256, 0, s>>>(planes, plane, pitch,
-                                                                         nx, ny, nplanes);
+    launch_dependent(k_periodic_T_x, nblk(int64_t(ny + 2) * nplanes, 256), 256, 0, s, planes,
+                     plane, pitch, nx, ny, nplanes);
   if (yper)
-    k_periodic_T_y<<<nblk(int64_t(xper ? nx : nx + 2) * nplanes, 256), 256, 0, s>>>(
-        planes, plane, pitch, nx, ny, nplanes, xper);
+    launch_dependent(k_periodic_T_y, nblk(int64_t(xper ? nx : nx + 2) * nplanes, 256), 256, 0, s,
+                     planes, plane, pitch, nx, ny, nplanes, xper);
   return cudaGetLastError();
 }
 
 cudaError_t launch_walls_T(const WallArgs& wa, float* lam, double* gtw, cudaStream_t s) {
   const int chunks = wall_chunk_count(wa.nseg, wa.seg);
   if (chunks == 0) return cudaSuccess;
-  k_walls_T<<<chunks, 32 * kWallWarpsT, 0, s>>>(wa, lam, gtw);
+  launch_dependent(k_walls_T, chunks, 32 * kWallWarpsT, 0, s, wa, lam, gtw);
   return cudaGetLastError();
 }
 

@@ -195,6 +195,7 @@ __global__ void __maxnreg__(128)
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  step_waits();
   __syncthreads();
   if (nrows <= 0) return;
 
@@ -222,6 +223,7 @@ __global__ void __maxnreg__(128)
       }
       tma_load_3d(stage + kBoxLSlot, &tape_map, col0, row0, d.z_tape, &full[st]);
     }
+    step_ends();
     return;
   }
 
@@ -323,9 +325,10 @@ cudaError_t launch_adj_tma(const AdjArgs& a, const void* lam_map, const void* la
   const dim3 block(32, kAW + 1);
   const dim3 grid((kX0 + a.nx - kAC0) / kATW + 1, (a.ny + 2 + kARows - 1) / kARows);
   if (adj_direct_ok(a, int(grid.x * grid.y))) return launch_adj_direct(a, order, s);
-  k_adj_tma<<<grid, block, adj_tma_bytes(a.q), s>>>(
-      a, *static_cast<const CUtensorMap*>(lam_map), *static_cast<const CUtensorMap*>(lam_map14),
-      *static_cast<const CUtensorMap*>(tape_map), tape_z0, order, status);
+  launch_dependent(k_adj_tma, grid, block, adj_tma_bytes(a.q), s, a,
+                   *static_cast<const CUtensorMap*>(lam_map),
+                   *static_cast<const CUtensorMap*>(lam_map14),
+                   *static_cast<const CUtensorMap*>(tape_map), tape_z0, order, status);
   return cudaGetLastError();
 }
 

@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(32 * kWallWarps) k_walls_batch(const BatchWall
 // values are the imposed ones relative to it (as for isothermal walls).
 template <typename T>
 __global__ void __launch_bounds__(256) k_sources(const SourceArgs a) {
+  step_waits();
   const int s = int(blockIdx.x) * 8 + (int(threadIdx.x) >> 5);
   const int lane = int(threadIdx.x) & 31;
   if (s >= a.n) return;
@@ -140,6 +141,7 @@ __device__ __forceinline__ void periodic_cell(const PeriodicArgs& a, int t, int 
 
 template <typename T>
 __global__ void k_periodic(const PeriodicArgs a) {
+  step_waits();
   periodic_cell<T>(a, int(blockIdx.x * blockDim.x + threadIdx.x), int(blockIdx.y));
 }
 
@@ -164,6 +166,7 @@ __global__ void __launch_bounds__(256) k_periodic_batch(const BatchInst* insts, 
   a.xper = I.a.xper; a.yper = I.a.yper;
   a.tape = 0;
   a.par = nullptr;
+  step_waits();
   periodic_cell<T>(a, (int(blockIdx.x) - at.y) * 256 + int(threadIdx.x), p);
 }
 
@@ -544,9 +547,9 @@ cudaError_t walls_t(const WallArgs& a, cudaStream_t s) {
   const int warps = staged ? staged_warps(a.q) : kWallWarps;
   const size_t bytes = staged ? size_t(a.q) * 32 * sizeof(float4) : 0;
   if (a.any_spec)
-    k_walls<T, true><<<chunks, 32 * warps, bytes, s>>>(a);
+    launch_dependent(k_walls<T, true>, chunks, 32 * warps, bytes, s, a);
   else
-    k_walls<T, false><<<chunks, 32 * warps, bytes, s>>>(a);
+    launch_dependent(k_walls<T, false>, chunks, 32 * warps, bytes, s, a);
   return cudaGetLastError();
 }
 
@@ -554,7 +557,9 @@ template <typename T>
 cudaError_t periodic_t(const PeriodicArgs& a, cudaStream_t s) {
   const int blocks = periodic_blocks(a.nx, a.ny, a.xper, a.yper);
   if (blocks == 0) return cudaSuccess;
-  k_periodic<T><<<dim3(unsigned(blocks), a.q + (a.e_ref ? 2 : 1)), 256, 0, s>>>(a);
+  const dim3 grid(unsigned(blocks), a.q + (a.e_ref ? 2 : 1));
+  if (int64_t(a.nx) * a.ny <= kEarlyPeriodicCells) launch_dependent(k_periodic<T>, grid, 256, 0, s, a);
+  else k_periodic<T><<<grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -567,14 +572,14 @@ int periodic_blocks(int nx, int ny, int xper, int yper) {
 }
 
 cudaError_t launch_periodic_batch(int storage, const BatchInst* insts, const int2* blocks,
-                                  int total_blocks, int max_q, int t, cudaStream_t s) {
+                                  int total_blocks, int max_q, bool early, int t,
+                                  cudaStream_t s) {
   if (total_blocks <= 0) return cudaSuccess;
-  if (storage == WLBM_STORE_BF16_DEV)
-    k_periodic_batch<__nv_bfloat16>
-        <<<dim3(unsigned(total_blocks), unsigned(max_q) + 2), 256, 0, s>>>(insts, blocks, t);
-  else
-    k_periodic_batch<float>
-        <<<dim3(unsigned(total_blocks), unsigned(max_q) + 1), 256, 0, s>>>(insts, blocks, t);
+  const bool bf = storage == WLBM_STORE_BF16_DEV;
+  const dim3 grid(unsigned(total_blocks), unsigned(max_q) + (bf ? 2 : 1));
+  const auto k = bf ? k_periodic_batch<__nv_bfloat16> : k_periodic_batch<float>;
+  if (early) launch_dependent(k, grid, 256, 0, s, insts, blocks, t);
+  else k<<<grid, 256, 0, s>>>(insts, blocks, t);
   return cudaGetLastError();
 }
 
@@ -583,11 +588,11 @@ cudaError_t launch_walls_batch(int storage, const BatchWalls* b, const int* bloc
   if (total_blocks <= 0) return cudaSuccess;
   const dim3 g{unsigned(total_blocks)}, blk{32 * kWallWarps};
   if (storage == WLBM_STORE_BF16_DEV) {
-    if (any_spec) k_walls_batch<__nv_bfloat16, true><<<g, blk, 0, s>>>(b, block_inst, t);
-    else k_walls_batch<__nv_bfloat16, false><<<g, blk, 0, s>>>(b, block_inst, t);
+    if (any_spec) launch_dependent(k_walls_batch<__nv_bfloat16, true>, g, blk, 0, s, b, block_inst, t);
+    else launch_dependent(k_walls_batch<__nv_bfloat16, false>, g, blk, 0, s, b, block_inst, t);
   } else {
-    if (any_spec) k_walls_batch<float, true><<<g, blk, 0, s>>>(b, block_inst, t);
-    else k_walls_batch<float, false><<<g, blk, 0, s>>>(b, block_inst, t);
+    if (any_spec) launch_dependent(k_walls_batch<float, true>, g, blk, 0, s, b, block_inst, t);
+    else launch_dependent(k_walls_batch<float, false>, g, blk, 0, s, b, block_inst, t);
   }
   return cudaGetLastError();
 }
@@ -651,9 +656,9 @@ cudaError_t launch_sources(int storage, const SourceArgs& a, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   const unsigned g = unsigned((a.n + 7) / 8);
   if (storage == WLBM_STORE_BF16_DEV)
-    k_sources<__nv_bfloat16><<<g, 256, 0, s>>>(a);
+    launch_dependent(k_sources<__nv_bfloat16>, g, 256, 0, s, a);
   else
-    k_sources<float><<<g, 256, 0, s>>>(a);
+    launch_dependent(k_sources<float>, g, 256, 0, s, a);
   return cudaGetLastError();
 }
 

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kThreads) k_step_direct(const StepArgs a) {
     d.own = paused ? int16_t(0) : d.from;
     table[j] = d;
   }
+  step_waits();
 #pragma unroll
   for (int h = 0; h < (kTile + kThreads - 1) / kThreads; ++h) {
     const int idx = tid + h * kThreads;
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(kThreads) k_step_direct(const StepArgs a) {
       if (REF) accw += d.w;
     }
   }
+  step_ends();
   a.e_out[cell] = REF ? fmaf(acc, a.scale, __fmul_rn(ein, accw)) : acc;
 }
 
@@ -217,6 +219,7 @@ __global__ void __launch_bounds__(kAdjThreads, 2) k_adj_direct(const AdjArgs a,
         out[d.plane] = keep * av;
       }
     }
+    step_ends();
     a.s_out[cell] = W * sigma;
     a.gw[cell] += fmaf(sigma - a0, ed, -pd);
     if (harvest) hrow[col == kGhostCol ? 0 : 1][ty] = hs;
@@ -235,8 +238,8 @@ template <typename T>
 cudaError_t launch_direct_t(const StepArgs& a, cudaStream_t s) {
   const dim3 grid((a.cmax - a.cmin) / 32 + 1, (a.rmax - a.rmin) / kRows + 1);
   const size_t bytes = size_t(a.q) * sizeof(DirectDir);
-  if (a.wfield) k_step_direct<T, true><<<grid, kThreads, bytes, s>>>(a);
-  else k_step_direct<T, false><<<grid, kThreads, bytes, s>>>(a);
+  if (a.wfield) launch_dependent(k_step_direct<T, true>, grid, kThreads, bytes, s, a);
+  else launch_dependent(k_step_direct<T, false>, grid, kThreads, bytes, s, a);
   return cudaGetLastError();
 }
 
@@ -267,7 +270,7 @@ bool adj_direct_ok(const AdjArgs& a, int tiles) {
 
 cudaError_t launch_adj_direct(const AdjArgs& a, const uint16_t* order, cudaStream_t s) {
   const dim3 grid((a.nx + 2 + 31) / 32, (a.ny + 2 + kAdjTmaRows - 1) / kAdjTmaRows);
-  k_adj_direct<<<grid, kAdjThreads, size_t(a.q) * sizeof(DirectAdj), s>>>(a, order);
+  launch_dependent(k_adj_direct, grid, kAdjThreads, size_t(a.q) * sizeof(DirectAdj), s, a, order);
   return cudaGetLastError();
 }
 

@@ -178,15 +178,15 @@ cudaError_t launch_tma_t(const StepArgs& a, const CUtensorMap& tm, cudaStream_t 
     const int ntiles = int(grid.x * grid.y);
     const int nb = std::min(a.loop_blocks, ntiles);
     if (a.wfield)
-      k_step_tma_loop<T, S, true, REF><<<nb, 32 * (kWarps3 + 1), bytes, s>>>(a, tm, int(grid.x),
-                                                                             ntiles);
+      launch_dependent(k_step_tma_loop<T, S, true, REF>, nb, 32 * (kWarps3 + 1), bytes, s, a, tm,
+                       int(grid.x), ntiles);
     else
-      k_step_tma_loop<T, S, false, REF><<<nb, 32 * (kWarps3 + 1), bytes, s>>>(a, tm, int(grid.x),
-                                                                              ntiles);
+      launch_dependent(k_step_tma_loop<T, S, false, REF>, nb, 32 * (kWarps3 + 1), bytes, s, a, tm,
+                       int(grid.x), ntiles);
     return cudaGetLastError();
   }
-  if (a.wfield) k_step_tma<T, S, true, REF><<<grid, block, bytes, s>>>(a, tm);
-  else k_step_tma<T, S, false, REF><<<grid, block, bytes, s>>>(a, tm);
+  if (a.wfield) launch_dependent(k_step_tma<T, S, true, REF>, grid, block, bytes, s, a, tm);
+  else launch_dependent(k_step_tma<T, S, false, REF>, grid, block, bytes, s, a, tm);
   return cudaGetLastError();
 }
 
@@ -238,8 +238,8 @@ cudaError_t launch_cells_t(const StepArgs& a, const CUtensorMap& tm, cudaStream_
   const dim3 block(32, kWarps3 + 1);
   const dim3 grid((a.cmax - a.cbase) / kTW3 + 1, (a.rmax - a.rmin + kRows3) / kRows3);
   const size_t bytes = TmaLayout<__nv_bfloat16, S>::bytes(a.q);
-  if (a.wfield) k_step_tma_cells<S, true><<<grid, block, bytes, s>>>(a, tm);
-  else k_step_tma_cells<S, false><<<grid, block, bytes, s>>>(a, tm);
+  if (a.wfield) launch_dependent(k_step_tma_cells<S, true>, grid, block, bytes, s, a, tm);
+  else launch_dependent(k_step_tma_cells<S, false>, grid, block, bytes, s, a, tm);
   return cudaGetLastError();
 }
 
@@ -271,8 +271,8 @@ int wide_cbase(const StepArgs& a) { return a.cmin < kX0 ? kX0 - 8 : kX0; }
 template <int S>
 cudaError_t launch_batch_wide_t(const BatchInst* insts, const int* tile_inst, int max_q,
                                 int total_tiles, int t, cudaStream_t s) {
-  k_step_tma_batch_wide<S><<<total_tiles, dim3(32, kWWarps + 1), WideLayout<S>::bytes(max_q),
-                             s>>>(insts, tile_inst, t);
+  launch_dependent(k_step_tma_batch_wide<S>, total_tiles, dim3(32, kWWarps + 1),
+                   WideLayout<S>::bytes(max_q), s, insts, tile_inst, t);
   return cudaGetLastError();
 }
 
@@ -282,8 +282,8 @@ cudaError_t launch_wide_t(const StepArgs& a, const CUtensorMap& tm, cudaStream_t
   const int cbase = wide_cbase(a);
   const dim3 grid((a.cmax - cbase) / kWTW + 1, (a.rmax - a.rmin + kRows3) / kRows3);
   const size_t bytes = WideLayout<S>::bytes(a.q);
-  if (a.wfield) k_step_tma_wide<S, true><<<grid, block, bytes, s>>>(a, tm, cbase);
-  else k_step_tma_wide<S, false><<<grid, block, bytes, s>>>(a, tm, cbase);
+  if (a.wfield) launch_dependent(k_step_tma_wide<S, true>, grid, block, bytes, s, a, tm, cbase);
+  else launch_dependent(k_step_tma_wide<S, false>, grid, block, bytes, s, a, tm, cbase);
   return cudaGetLastError();
 }
 
@@ -308,12 +308,12 @@ cudaError_t launch_step_tma_batch(int storage, const BatchInst* insts,
   const dim3 block(32, kWarps3 + 1);
   if (storage == WLBM_STORE_BF16_DEV) {
     using LY = TmaLayout<__nv_bfloat16, kStagesBF16>;
-    k_step_tma_batch<__nv_bfloat16, kStagesBF16, true>
-        <<<total_tiles, block, LY::bytes(max_q), s>>>(insts, tile_inst, t);
+    launch_dependent(k_step_tma_batch<__nv_bfloat16, kStagesBF16, true>, total_tiles, block,
+                     LY::bytes(max_q), s, insts, tile_inst, t);
   } else {
     using LY = TmaLayout<float, kStagesF32>;
-    k_step_tma_batch<float, kStagesF32, false>
-        <<<total_tiles, block, LY::bytes(max_q), s>>>(insts, tile_inst, t);
+    launch_dependent(k_step_tma_batch<float, kStagesF32, false>, total_tiles, block,
+                     LY::bytes(max_q), s, insts, tile_inst, t);
   }
   return cudaGetLastError();
 }

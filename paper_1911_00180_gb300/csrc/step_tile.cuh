@@ -840,6 +840,7 @@ __device__ __forceinline__ bool step_tma_tile(const StepArgs& a, const void* tma
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (!PERSIST) step_waits();
   __syncthreads();
   if (nrows <= 0) return true;
   uint32_t g = PERSIST ? g0 : 0u;
@@ -852,7 +853,9 @@ __device__ __forceinline__ bool step_tma_tile(const StepArgs& a, const void* tma
     // and the ring by this block's wall chunks; order the tensor copies after those
     // generic-proxy writes
     if (PERSIST) asm volatile("fence.proxy.async;" ::: "memory");
-    return produce_tile<T, S>(a, tmap, col0, row0, g, m);
+    const bool ok = produce_tile<T, S>(a, tmap, col0, row0, g, m);
+    if (!PERSIST) step_ends();
+    return ok;
   }
   // ---------------------------------------------------------------- consumer warps
   if constexpr (REF && CELLS) {
@@ -891,6 +894,7 @@ __device__ __forceinline__ void step_tma_loop(const StepArgs& a, const void* tma
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *fail = 0;
   }
+  step_waits();
   __syncthreads();
   uint32_t g = 0;
   const int first = int(blockIdx.x), stride = int(gridDim.x);

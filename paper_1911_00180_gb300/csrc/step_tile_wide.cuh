@@ -75,6 +75,7 @@ __device__ __forceinline__ void step_tma_tile_wide(const StepArgs& a, const void
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  step_waits();
   __syncthreads();
   if (nrows <= 0) return;
 
@@ -94,6 +95,7 @@ __device__ __forceinline__ void step_tma_tile_wide(const StepArgs& a, const void
       tma_load_3d(smem + st * LY::kStage, tmap, (col0 - 8) / 2, row0 + (d.zdy & 3) - 1,
                   d.zdy >> 2, &full[st]);
     }
+    step_ends();
     return;
   }
 

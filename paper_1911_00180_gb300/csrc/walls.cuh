@@ -303,6 +303,7 @@ __device__ __forceinline__ void walls_chunk(const WallArgs& a, const uint8_t* co
     sm.rho[i] = diffuse ? rho[i] : 0.f;
     if (SPEC) sm.src[i] = diffuse && g.spec > 0.f ? mir[i] : int16_t(i);
   }
+  step_waits();
   __syncthreads();
   if (!wall_seg_rowwise(g)) {                  // one warp per cell, lanes over directions
     const int cell = c * kWallCellsPerBlock + warp;

@@ -1783,6 +1783,7 @@ struct wlbm_batch {
   std::vector<int> per;             // instances whose periodic edges need the separate pass
   int2* d_per = nullptr;            // {instance, its first block column} of every block column
   int per_cap = 0, per_blocks = 0, per_q = 0;   // of that pass; the largest Q among them
+  int64_t per_cells = 0;            // cells of those instances
   // A captured chunk (the batched kernels read planes and phases at run time), two for the
   // replay parities, as for a single grid.
   TimedGraph graphs[2];
@@ -1868,11 +1869,13 @@ struct wlbm_batch {
     per.clear();
     std::vector<int2> blocks;
     per_q = 0;
+    per_cells = 0;
     for (size_t k = 0; k < h.size(); ++k) {
       const wlbm_handle* x = h[k];
       if (!(x->xper || x->yper) || wraps(x)) continue;
       per.push_back(int(k));
       per_q = std::max(per_q, x->g.q);
+      per_cells += int64_t(x->g.nx) * x->g.ny;
       const int first = int(blocks.size());
       blocks.insert(blocks.end(), size_t(periodic_blocks(x->g.nx, x->g.ny, x->xper, x->yper)),
                     make_int2(int(k), first));
@@ -2237,8 +2240,8 @@ static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every, TimedGraph
       ++b->launches;
     }
     if (st == WLBM_OK && b->per_blocks > 0) {
-      st = b->cuda(launch_periodic_batch(b->storage, b->d_inst, b->d_per, b->per_blocks, b->per_q, t,
-                                         b->stream), "wlbm_batch_step: periodic");
+      st = b->cuda(launch_periodic_batch(b->storage, b->d_inst, b->d_per, b->per_blocks, b->per_q,
+                                         b->per_cells <= kEarlyPeriodicCells, t, b->stream), "wlbm_batch_step: periodic");
       ++b->launches;
     }
     if (st != WLBM_OK) break;

@@ -125,6 +125,25 @@ inline void sort_by_kind(const uint8_t* codes, int q, uint16_t* out) {
 }
 
 #ifdef __CUDACC__
+// Launch a kernel of a step as a programmatic dependent of the kernel ahead of it in the
+// stream (step_ends / step_waits in elem.cuh; behind anything but a kernel this is an
+// ordinary launch).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Uniform W_corr of a frame cell: w0 inside the frame, 0 on pads and on the ghost cells of
 // walls (wall cells do not scatter); periodic ghost cells carry w0.
 __device__ __forceinline__ float uniform_w(const StepArgs& a, int r, int c) {
@@ -198,6 +217,12 @@ __host__ __device__ inline int wall_chunk_segment(int nseg, const WallSeg* seg, 
 }
 #endif
 
+
+// Periodic passes of up to this many cells start as dependents of the step ahead of them; on
+// larger grids their waiting blocks cost the step's last waves more than the early start gives
+// (early / not, us a step: 512^2 x Q64 27.1 / 27.9, 1024^2 x Q64 99.9 / 100.4, 1400^2 x Q32
+// 89.4 / 89.5, 2048^2 x Q16 99.1 / 98.4, 2048^2 x Q64 341.2 / 338.6, bfloat16 194.5 / 191.8).
+constexpr int64_t kEarlyPeriodicCells = int64_t(1) << 21;
 
 struct PeriodicArgs {
   void* planes;
@@ -477,7 +502,8 @@ cudaError_t launch_periodic(int storage, const PeriodicArgs& a, cudaStream_t s);
 // the largest Q among them.
 int periodic_blocks(int nx, int ny, int xper, int yper);
 cudaError_t launch_periodic_batch(int storage, const BatchInst* insts, const int2* blocks,
-                                  int total_blocks, int max_q, int t, cudaStream_t s);
+                                  int total_blocks, int max_q, bool early, int t,
+                                  cudaStream_t s);
 // Smallest and largest of n floats (NaN left out) as ordered bits into out[0], out[1]; the
 // value of such bits (false: none, every float was NaN).
 cudaError_t launch_range(const float* x, int64_t n, unsigned* out, cudaStream_t s);
