@@ -356,9 +356,22 @@ __global__ void k_adj_seed(const AdjArgs a, const float* dJ_dT, const float* dJ_
     a.lam_out[int64_t(i) * a.plane + off] = fmaf(gy, sy[i], fmaf(gx, sx[i], g));
 }
 
+// dW_corr/dMFP (Eq. W-correction with W = v/MFP: a function of m = MFP/v, so dW_corr/dMFP =
+// (dW_corr/dm) / v).  Rounded operation by operation: a fused one would give other bits.
+__device__ __forceinline__ float dw_dmfp(const AdjMfp& a, int cell) {
+  const double m = __ddiv_rn(a.mfp ? double(a.mfp[cell]) : a.uniform, a.speed);
+  if (isinf(m)) return 0.f;
+  const double W = __ddiv_rn(1.0, m), l1 = __dadd_rn(a.lam_corr, -1.0);
+  double d = __ddiv_rn(
+      __dmul_rn(-a.f, __dadd_rn(1.0, __dmul_rn(__dmul_rn(2.0, W), l1))), __dmul_rn(m, m));
+  if (a.relax_mode == 1)
+    d = __dmul_rn(d, exp(__dmul_rn(-a.f, __dadd_rn(W, __dmul_rn(__dmul_rn(W, W), l1)))));
+  return float(__ddiv_rn(d, a.speed));
+}
+
 // dJ/dMFP = dJ/dW_corr * dW_corr/dMFP on interior cells; dJ/d(dT0) from l^0 through the
 // initial condition e_i = w_i e_eq(T_ref + dT0) (ghost cells copy the nearest cell).
-__global__ void k_adj_final(const AdjArgs a, const float* dwc, float* dJ_dmfp,
+__global__ void k_adj_final(const AdjArgs a, const AdjMfp mf, float* dJ_dmfp,
                             const float* lam0, const float* s0, const float* dT0,
                             float* dJ_ddT0, double t_ref, double theta) {
   // weights as float64, and their sum, once a block: the float64 pipe bounds this kernel
@@ -376,7 +389,7 @@ __global__ void k_adj_final(const AdjArgs a, const float* dwc, float* dJ_dmfp,
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nx * a.ny) return;
   const int y = t / a.nx, x = t - y * a.nx;
-  if (dJ_dmfp) dJ_dmfp[t] = a.gw[int64_t(y + 2) * a.pitch + (x + kX0)] * dwc[t];
+  if (dJ_dmfp) dJ_dmfp[t] = a.gw[int64_t(y + 2) * a.pitch + (x + kX0)] * dw_dmfp(mf, t);
   if (dJ_ddT0) {
     const int fx[3] = {x, x == 0 ? -1 : x, x == a.nx - 1 ? a.nx : x};
     const int fy[3] = {y, y == 0 ? -1 : y, y == a.ny - 1 ? a.ny : y};
@@ -436,10 +449,10 @@ cudaError_t launch_adj_seed(const AdjArgs& a, const float* dJ_dT, const float* d
   return cudaGetLastError();
 }
 
-cudaError_t launch_adj_final(const AdjArgs& a, const float* dwc, float* dJ_dmfp,
+cudaError_t launch_adj_final(const AdjArgs& a, const AdjMfp& mf, float* dJ_dmfp,
                              const float* lam0, const float* s0, const float* dT0,
                              float* dJ_ddT0, double t_ref, double theta, cudaStream_t s) {
-  k_adj_final<<<nblk(int64_t(a.nx) * a.ny, 256), 256, 0, s>>>(a, dwc, dJ_dmfp, lam0, s0, dT0,
+  k_adj_final<<<nblk(int64_t(a.nx) * a.ny, 256), 256, 0, s>>>(a, mf, dJ_dmfp, lam0, s0, dT0,
                                                                dJ_ddT0, t_ref, theta);
   return cudaGetLastError();
 }

@@ -179,7 +179,7 @@ struct wlbm_handle {
     float* sh[2] = {nullptr, nullptr};    // shared part s (one plane)
     float* erec[2] = {nullptr, nullptr};
     float* gw = nullptr;       // framed dJ/dW_corr
-    float* dwc = nullptr;      // nx*ny dW_corr/dMFP
+    float* mfp = nullptr;      // nx*ny mean free paths (grids with a field)
     float* dT0 = nullptr;      // nx*ny start field
     double* gtw = nullptr;     // [4] sum_i w_i lambda_i at isothermal ghosts
     uint8_t* codes = nullptr;  // [n][q] schedule of the run
@@ -1487,14 +1487,14 @@ static wlbm_status adj_alloc(wlbm_handle* h, int64_t n, int k) {
   A.erec[0] = static_cast<float*>(get(size_t(g.plane) * 4));
   A.erec[1] = static_cast<float*>(get(size_t(g.plane) * 4));
   A.gw = static_cast<float*>(get(size_t(g.plane) * 4));
-  A.dwc = static_cast<float*>(get(cells));
+  A.mfp = h->field_w ? static_cast<float*>(get(cells)) : nullptr;
   A.dT0 = static_cast<float*>(get(cells));
   A.gtw = static_cast<double*>(get(4 * sizeof(double)));
   A.codes = static_cast<uint8_t*>(get(size_t(n) * g.q));
   A.order = static_cast<uint16_t*>(get(size_t(n) * (g.q + 17) * 2));
   if (!A.ckpt || !A.ckpt_e || !A.tape || !A.lam[0] || !A.lam[1] || !A.sh[0] || !A.sh[1] ||
       !A.erec[0] || !A.erec[1] ||
-      !A.gw || !A.dwc || !A.dT0 || !A.gtw || !A.codes || !A.order)
+      !A.gw || (h->field_w && !A.mfp) || !A.dT0 || !A.gtw || !A.codes || !A.order)
     return h->fail(WLBM_ERR_OOM, "wlbm_adjoint_forward: device allocation failed");
   A.n = n;
   A.k = k;
@@ -1516,6 +1516,8 @@ static wlbm_status adj_alloc(wlbm_handle* h, int64_t n, int k) {
   cudaError_t e = cudaMemsetAsync(tape_raw, 0, size_t(k) * state + 1024, h->stream);
   for (int j = 0; j < 2 && e == cudaSuccess; ++j)
     e = cudaMemsetAsync(A.erec[j], 0, size_t(g.plane) * 4, h->stream);
+  if (e == cudaSuccess && A.mfp)
+    e = cudaMemcpyAsync(A.mfp, h->mfp_host.data(), cells, cudaMemcpyHostToDevice, h->stream);
   return h->cuda(e, "wlbm_adjoint_forward");
 }
 
@@ -1534,18 +1536,6 @@ wlbm_status wlbm_adjoint_forward(wlbm_handle* h, const float* dT0, int64_t n_ste
   if (!(A.n == n_steps && A.k == ckpt_every && A.ckpt)) st = adj_alloc(h, n_steps, ckpt_every);
   if (st != WLBM_OK) return st;
   A.ready = false;
-  // dW_corr/dMFP per interior cell (Eq. W-correction with W = v/MFP: a function of
-  // m = MFP/v, so dW_corr/dMFP = (dW_corr/dm) / v)
-  std::vector<float> dwc(size_t(g.nx) * g.ny);
-  const double f = h->emulate_3d ? 1.5 : 1.0, lc = h->lat.lam_corr, v = h->lat.speed;
-  for (size_t c = 0; c < dwc.size(); ++c) {
-    const double m = (h->field_w ? double(h->mfp_host[c]) : h->mfp_uniform) / v;
-    if (std::isinf(m)) { dwc[c] = 0.f; continue; }
-    const double W = 1.0 / m;
-    double d = -f * (1.0 + 2.0 * W * (lc - 1.0)) / (m * m);
-    if (h->relax_mode == 1) d *= std::exp(-f * (W + W * W * (lc - 1.0)));
-    dwc[c] = float(d / v);
-  }
   std::vector<uint8_t> codes(size_t(n_steps) * g.q);
   std::vector<uint16_t> order(size_t(n_steps) * (g.q + 17));
   TasState ts;
@@ -1555,11 +1545,8 @@ wlbm_status wlbm_adjoint_forward(wlbm_handle* h, const float* dT0, int64_t n_ste
     sort_by_kind(codes.data() + t * g.q, g.q, order.data() + t * (g.q + 17));
   }
   cudaStream_t s = h->stream;
-  st = h->cuda(cudaMemcpyAsync(A.dwc, dwc.data(), dwc.size() * 4, cudaMemcpyHostToDevice, s),
+  st = h->cuda(cudaMemcpyAsync(A.codes, codes.data(), codes.size(), cudaMemcpyHostToDevice, s),
                "wlbm_adjoint_forward");
-  if (st == WLBM_OK)
-    st = h->cuda(cudaMemcpyAsync(A.codes, codes.data(), codes.size(), cudaMemcpyHostToDevice, s),
-                 "wlbm_adjoint_forward");
   if (st == WLBM_OK)
     st = h->cuda(cudaMemcpyAsync(A.order, order.data(), order.size() * 2, cudaMemcpyHostToDevice,
                                  s), "wlbm_adjoint_forward");
@@ -1711,7 +1698,10 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
   // periodic ghosts of W_corr copy interior cells: send their gradient back
   ok(launch_periodic_T(A.gw, g.plane, g.pitch, g.nx, g.ny, 1, h->xper, h->yper, s),
      "adjoint: W transpose");
-  ok(launch_adj_final(aa, A.dwc, dJ_dmfp, A.lam[cur], A.sh[cur], A.dT0, dJ_ddT0, h->t_ref,
+  AdjMfp mf{};
+  mf.mfp = A.mfp; mf.uniform = h->mfp_uniform; mf.speed = h->lat.speed;
+  mf.lam_corr = h->lat.lam_corr; mf.f = h->emulate_3d ? 1.5 : 1.0; mf.relax_mode = h->relax_mode;
+  ok(launch_adj_final(aa, mf, dJ_dmfp, A.lam[cur], A.sh[cur], A.dT0, dJ_ddT0, h->t_ref,
                       h->theta, s),
      "adjoint: final");
   double gt[4] = {0, 0, 0, 0};

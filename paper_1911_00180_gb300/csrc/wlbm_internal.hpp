@@ -394,6 +394,13 @@ struct AdjArgs {
   double* gtw;
 };
 
+// Mean free paths and what W_corr depends on besides them, for dW_corr/dMFP.
+struct AdjMfp {
+  const float* mfp;      // nx*ny, or nullptr (uniform)
+  double uniform, speed, lam_corr, f;   // f: 3/2 (3-D emulation) or 1
+  int relax_mode;
+};
+
 #ifdef __CUDACC__
 // W_corr of frame cell (r, c) for the reverse step: the framed field, or w0 by the frame
 // rule (pads and wall ghosts 0).
@@ -541,7 +548,7 @@ cudaError_t launch_sources(int storage, const SourceArgs& a, cudaStream_t s);
 cudaError_t launch_adj_seed(const AdjArgs& a, const float* dJ_dT, const float* dJ_dqx,
                             const float* dJ_dqy, const float* sx, const float* sy, float vg,
                             const float* e_final, double e_ref, double theta, cudaStream_t s);
-cudaError_t launch_adj_final(const AdjArgs& a, const float* dwc, float* dJ_dmfp,
+cudaError_t launch_adj_final(const AdjArgs& a, const AdjMfp& mf, float* dJ_dmfp,
                              const float* lam0, const float* s0, const float* dT0,
                              float* dJ_ddT0, double t_ref, double theta, cudaStream_t s);
 
