@@ -177,14 +177,16 @@ __global__ void __launch_bounds__(32 * kAdjRows) k_adj_step(const AdjArgs a) {
     atomicAdd(a.gtw + tid, double(hwall[tid]));
 }
 
-// Transpose of the periodic x link (all frame rows), then of the y link.
-__global__ void k_periodic_T_x(float* planes, int64_t plane, int pitch, int nx, int ny,
-                               int nplanes) {
+// Transpose of the periodic x link (all frame rows), then of the y link, on the direction planes
+// and, as one plane more, on `shared` (one launch for both: 3.4 us less a reverse step of
+// 1024^2 x Q64).
+__global__ void k_periodic_T_x(float* planes, float* shared, int64_t plane, int pitch, int nx,
+                               int ny, int nplanes) {
   step_waits();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (ny + 2) * nplanes) return;
+  if (t >= (ny + 2) * (nplanes + (shared ? 1 : 0))) return;
   const int p = t / (ny + 2), r = 1 + (t - p * (ny + 2));
-  float* row = planes + int64_t(p) * plane + int64_t(r) * pitch;
+  float* row = (p < nplanes ? planes + int64_t(p) * plane : shared) + int64_t(r) * pitch;
   const float gl = row[kGhostCol], gr = row[kX0 + nx];
   row[kX0 + nx - 1] += gl;
   row[kX0] += gr;
@@ -192,14 +194,14 @@ __global__ void k_periodic_T_x(float* planes, int64_t plane, int pitch, int nx, 
   row[kX0 + nx] = 0.f;
 }
 
-__global__ void k_periodic_T_y(float* planes, int64_t plane, int pitch, int nx, int ny,
-                               int nplanes, int xper) {
+__global__ void k_periodic_T_y(float* planes, float* shared, int64_t plane, int pitch, int nx,
+                               int ny, int nplanes, int xper) {
   step_waits();
   const int ncol = xper ? nx : nx + 2, c0 = xper ? kX0 : kGhostCol;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ncol * nplanes) return;
+  if (t >= ncol * (nplanes + (shared ? 1 : 0))) return;
   const int p = t / ncol, c = c0 + (t - p * ncol);
-  float* base = planes + int64_t(p) * plane + c;
+  float* base = (p < nplanes ? planes + int64_t(p) * plane : shared) + c;
   const float gb = base[int64_t(1) * pitch], gt = base[int64_t(ny + 2) * pitch];
   base[int64_t(ny + 1) * pitch] += gb;
   base[int64_t(2) * pitch] += gt;
@@ -423,14 +425,15 @@ cudaError_t launch_adj_step(const AdjArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_periodic_T(float* planes, int64_t plane, int pitch, int nx, int ny,
-                              int nplanes, int xper, int yper, cudaStream_t s) {
+cudaError_t launch_periodic_T(float* planes, float* shared, int64_t plane, int pitch, int nx,
+                              int ny, int nplanes, int xper, int yper, cudaStream_t s) {
+  const int all = nplanes + (shared ? 1 : 0);
   if (xper)
-    launch_dependent(k_periodic_T_x, nblk(int64_t(ny + 2) * nplanes, 256), 256, 0, s, planes,
+    launch_dependent(k_periodic_T_x, nblk(int64_t(ny + 2) * all, 256), 256, 0, s, planes, shared,
                      plane, pitch, nx, ny, nplanes);
   if (yper)
-    launch_dependent(k_periodic_T_y, nblk(int64_t(xper ? nx : nx + 2) * nplanes, 256), 256, 0, s,
-                     planes, plane, pitch, nx, ny, nplanes, xper);
+    launch_dependent(k_periodic_T_y, nblk(int64_t(xper ? nx : nx + 2) * all, 256), 256, 0, s,
+                     planes, shared, plane, pitch, nx, ny, nplanes, xper);
   return cudaGetLastError();
 }
 

@@ -1682,10 +1682,8 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
       else
         ok(launch_adj_step(aa, s), "adjoint: reverse step");
       // the periodic transpose is the same on every direction: it acts on lh and on s
-      ok(launch_periodic_T(A.lam[cur ^ 1], g.plane, g.pitch, g.nx, g.ny, g.q, h->xper, h->yper, s),
-         "adjoint: periodic transpose");
-      ok(launch_periodic_T(A.sh[cur ^ 1], g.plane, g.pitch, g.nx, g.ny, 1, h->xper, h->yper, s),
-         "adjoint: periodic transpose");
+      ok(launch_periodic_T(A.lam[cur ^ 1], A.sh[cur ^ 1], g.plane, g.pitch, g.nx, g.ny, g.q,
+                           h->xper, h->yper, s), "adjoint: periodic transpose");
       // s is zero on wall ghost cells (W = 0 there), so the wall transpose sees l = lh
       if (h->walls.nseg > 0) {
         WallArgs wa = h->walls;
@@ -1696,7 +1694,7 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
     }
   }
   // periodic ghosts of W_corr copy interior cells: send their gradient back
-  ok(launch_periodic_T(A.gw, g.plane, g.pitch, g.nx, g.ny, 1, h->xper, h->yper, s),
+  ok(launch_periodic_T(A.gw, nullptr, g.plane, g.pitch, g.nx, g.ny, 1, h->xper, h->yper, s),
      "adjoint: W transpose");
   AdjMfp mf{};
   mf.mfp = A.mfp; mf.uniform = h->mfp_uniform; mf.speed = h->lat.speed;

@@ -522,8 +522,8 @@ cudaError_t launch_get_state(int storage, const StateArgs& a, cudaStream_t s);
 cudaError_t launch_set_state(int storage, const StateArgs& a, cudaStream_t s);
 // Adjoint launchers (k_adjoint.cu).
 cudaError_t launch_adj_step(const AdjArgs& a, cudaStream_t s);
-cudaError_t launch_periodic_T(float* planes, int64_t plane, int pitch, int nx, int ny,
-                              int nplanes, int xper, int yper, cudaStream_t s);
+cudaError_t launch_periodic_T(float* planes, float* shared, int64_t plane, int pitch, int nx,
+                              int ny, int nplanes, int xper, int yper, cudaStream_t s);
 // Transposed wall pass after the periodic transpose.  Isothermal cells were transposed by
 // the reverse step: only the two end cells of each isothermal segment (where the periodic
 // transpose of the other axis may have added corner images) are transposed again.
