@@ -265,14 +265,22 @@ __global__ void __launch_bounds__(256) k_init(const InitArgs a) {
   a.e_cur[off] = e;
 }
 
-// e_i - e_j of one cell from their stored values: float32 deviations subtract directly;
-// bfloat16 ones subtract before the scaling, and the reference parts w R leave only
-// (w_i - w_j) R.
-template <typename T>
-__device__ __forceinline__ float dev_diff(const T* pi, const T* pj, float wi, float wj,
-                                          const float* ref, int64_t off, float scale) {
-  const float d = Elem<T>::ld(pi) - Elem<T>::ld(pj);
-  return ref ? fmaf(d, scale, __fmul_rn(wi - wj, ref[off])) : d;
+// A pair of opposite directions i and j = i + Q/2 as the flux sums need it: the elements of
+// their current planes relative to the buffer, w_i - w_j and s_i.  Staged once a block, so that a
+// pair costs two loads and the arithmetic (parities, weights and plane offsets worked out per
+// cell kept the warps issuing, not loading).
+struct alignas(16) FluxPair {
+  int64_t i, j;
+  float dw, sx, sy, pad;
+};
+template <typename Par>
+__device__ __forceinline__ void stage_pairs(FluxPair* tab, int64_t plane, int q, Par par,
+                                            const float* w, const float* sx, const float* sy) {
+  for (int i = int(threadIdx.x); i < q / 2; i += int(blockDim.x)) {
+    const int j = i + q / 2;
+    tab[i] = {int64_t(par(i) * q + i) * plane, int64_t(par(j) * q + j) * plane, w[i] - w[j],
+              sx[i], sy[i], 0.f};
+  }
 }
 
 // Heat flux of one cell, q = sum_i e_i s_i (Eq. heat-flux, v = 1 here), taken over the
@@ -282,32 +290,57 @@ __device__ __forceinline__ float dev_diff(const T* pi, const T* pj, float wi, fl
 // the float32 result is within a few roundings of |q| for any Q, where a plain float32 sum
 // of Q products errs by about Q roundings of the summands' magnitude (at Q = 1024 more than
 // 1e-5 of a direction's amplitude).
-template <typename T, typename Par>
-__device__ __forceinline__ void cell_flux(const T* planes, int64_t plane, int q, Par par,
-                                          const float* w, const float* sx, const float* sy,
-                                          const float* ref, int64_t off, float scale,
-                                          float& qx, float& qy) {
-  const int h = q / 2;
+// The difference e_i - e_j of stored values: float32 deviations subtract directly; bfloat16 ones
+// before the scaling, and the reference parts w R leave only (w_i - w_j) R.  at: the cell's
+// element in the buffer; four pairs' values are loaded while the previous four are added.
+template <typename T>
+__device__ __forceinline__ void cell_flux(const T* at, const FluxPair* tab, int q, bool ref,
+                                          float R, float scale, float& qx, float& qy) {
+  const int h = q / 2;        // a multiple of 4
   float cx = 0.f, cy = 0.f;   // compensations: what the running sums lost
   qx = 0.f;
   qy = 0.f;
-#pragma unroll 4
-  for (int i = 0; i < h; ++i) {
-    const int j = i + h;
-    const float d = dev_diff(planes + int64_t(par(i) * q + i) * plane + off,
-                             planes + int64_t(par(j) * q + j) * plane + off, w[i], w[j], ref,
-                             off, scale);
-    const float yx = fmaf(d, sx[i], -cx), yy = fmaf(d, sy[i], -cy);
-    const float tx = qx + yx, ty = qy + yy;
-    cx = (tx - qx) - yx;
-    cy = (ty - qy) - yy;
-    qx = tx;
-    qy = ty;
+  float na[4], nb[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    na[u] = Elem<T>::ld(at + tab[u].i);
+    nb[u] = Elem<T>::ld(at + tab[u].j);
+  }
+  for (int i = 0; i < h; i += 4) {
+    float d[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) d[u] = na[u] - nb[u];
+    if (i + 4 < h) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        na[u] = Elem<T>::ld(at + tab[i + 4 + u].i);
+        nb[u] = Elem<T>::ld(at + tab[i + 4 + u].j);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const FluxPair p = tab[i + u];
+      const float v = ref ? fmaf(d[u], scale, __fmul_rn(p.dw, R)) : d[u];
+      const float yx = fmaf(v, p.sx, -cx), yy = fmaf(v, p.sy, -cy);
+      const float tx = qx + yx, ty = qy + yy;
+      cx = (tx - qx) - yx;
+      cy = (ty - qy) - yy;
+      qx = tx;
+      qy = ty;
+    }
   }
 }
 
+// Bound by the one read of the state: 4096 x 256 x Q128 91 us (126 with the per-direction data
+// worked out per cell), the copy rate's floor 80.
 template <typename T>
-__global__ void k_moments(const MomentArgs a) {
+__global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
+  extern __shared__ __align__(16) unsigned char pair_smem[];
+  FluxPair* tab = reinterpret_cast<FluxPair*>(pair_smem);
+  if (a.qx || a.qy) {
+    stage_pairs(tab, a.plane, a.q, [&](int i) { return parity_of(a.par, i); }, a.w, a.sx, a.sy);
+    __syncthreads();
+  }
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nx * a.ny) return;
   const int y = t / a.nx, x = t - y * a.nx;
@@ -322,9 +355,8 @@ __global__ void k_moments(const MomentArgs a) {
   }
   if (a.qx || a.qy) {
     float qx, qy;
-    cell_flux(static_cast<const T*>(a.planes), a.plane, a.q,
-              [&](int i) { return parity_of(a.par, i); }, a.w, a.sx, a.sy, a.e_refp, off,
-              a.scale, qx, qy);
+    cell_flux(static_cast<const T*>(a.planes) + off, tab, a.q, a.e_refp != nullptr,
+              a.e_refp ? a.e_refp[off] : 0.f, a.scale, qx, qy);
     const float wx = a.weight * (qx * a.vg), wy = a.weight * (qy * a.vg);
     if (a.qx) a.qx[t] = a.accumulate ? a.qx[t] + wx : wx;
     if (a.qy) a.qy[t] = a.accumulate ? a.qy[t] + wy : wy;
@@ -357,14 +389,15 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 
 // Per-direction data of a reduction block, staged once in shared memory.
 struct ReduceSmem {
-  float w[kMaxQ], sx[kMaxQ], sy[kMaxQ];
+  float w[kMaxQ];
   uint8_t par[kMaxQ];
 };
 
 // Per-cell contributions of k_reduce at framed index t: the sums v[] and the residual.
 template <typename T>
-__device__ __forceinline__ void reduce_cell(const ReduceArgs& a, const ReduceSmem& sm, int t,
-                                            double* v, double* res, double* resw) {
+__device__ __forceinline__ void reduce_cell(const ReduceArgs& a, const ReduceSmem& sm,
+                                            const FluxPair* tab, int t, double* v, double* res,
+                                            double* resw) {
   const int fw = a.nx + 2, fh = a.ny + 2;
   const int fy = t / fw, fx = t - fy * fw;
   const bool gx = fx == 0 || fx == fw - 1, gy = fy == 0 || fy == fh - 1;
@@ -377,8 +410,8 @@ __device__ __forceinline__ void reduce_cell(const ReduceArgs& a, const ReduceSme
     // a cell's flux over its Q directions in float32 (as in k_moments: the stored values
     // are float32 or coarser), the sums over cells in float64
     float qx, qy;
-    cell_flux(planes, a.plane, a.q, [&](int i) { return int(sm.par[i]); }, sm.w, sm.sx, sm.sy,
-              a.e_refp, off, float(a.scale), qx, qy);
+    cell_flux(planes + off, tab, a.q, a.e_refp != nullptr, a.e_refp ? a.e_refp[off] : 0.f,
+              float(a.scale), qx, qy);
     v[2] += qx;
     v[3] += qy;
     const int x = fx - 1;
@@ -410,64 +443,19 @@ __device__ __forceinline__ void reduce_cell(const ReduceArgs& a, const ReduceSme
   }
 }
 
-// Stage 1: a grid-stride pass; block b writes its kReduceOut partial results to
-// a.part[b] (no atomics: a second kernel combines the blocks in a fixed order).
-template <typename T>
-__global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
-  const int cells = (a.nx + 2) * (a.ny + 2);
-  __shared__ ReduceSmem sm;
-  for (int i = int(threadIdx.x); i < a.q; i += 256) {
-    sm.w[i] = a.w[i];
-    sm.sx[i] = a.sx[i];
-    sm.sy[i] = a.sy[i];
-    sm.par[i] = uint8_t(parity_of(a.par, i));
-  }
-  __syncthreads();
-  double v[kReduceSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  double res = 0.0, resw = 0.0;   // largest |T - T_snap| and window change (>= 0 or NaN)
-  for (int t = int(blockIdx.x) * 256 + int(threadIdx.x); t < cells; t += int(gridDim.x) * 256)
-    reduce_cell<T>(a, sm, t, v, &res, &resw);
-  __shared__ double red[kReduceSums][8];
-  __shared__ unsigned long long redm[2][8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kReduceSums; ++k) {
-    const double s = warp_sum(v[k]);
-    if (lane == 0) red[k][wid] = s;
-  }
-  // |.| is non-negative, so its bit pattern orders like its value (NaN above all)
-  const unsigned long long m0 = warp_max_u64(static_cast<unsigned long long>(__double_as_longlong(res)));
-  const unsigned long long m1 = warp_max_u64(static_cast<unsigned long long>(__double_as_longlong(resw)));
-  if (lane == 0) {
-    redm[0][wid] = m0;
-    redm[1][wid] = m1;
-  }
-  __syncthreads();
-  if (threadIdx.x < kReduceSums) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
-    a.part[int64_t(blockIdx.x) * kReduceOut + threadIdx.x] = s;
-  } else if (threadIdx.x < kReduceOut) {
-    unsigned long long m = 0ull;
-    for (int w = 0; w < 8; ++w) m = redm[threadIdx.x - kReduceSums][w] > m
-                                        ? redm[threadIdx.x - kReduceSums][w] : m;
-    a.part[int64_t(blockIdx.x) * kReduceOut + threadIdx.x] = __longlong_as_double(
-        static_cast<long long>(m));
-  }
-}
-
-// Stage 2, one block: the blocks' partials combined in a fixed order into a.out.
-__global__ void __launch_bounds__(256) k_reduce_finish(const ReduceArgs a, int nblocks) {
+// Stage 2, by the block that ends last: the blocks' partials combined in a fixed order into
+// a.out.
+__device__ __forceinline__ void reduce_finish(const ReduceArgs& a, int nblocks) {
   double v[kReduceSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   unsigned long long m[2] = {0ull, 0ull};
   for (int b = int(threadIdx.x); b < nblocks; b += 256) {
     const double* p = a.part + int64_t(b) * kReduceOut;
 #pragma unroll
-    for (int k = 0; k < kReduceSums; ++k) v[k] += p[k];
+    for (int k = 0; k < kReduceSums; ++k) v[k] += __ldcg(p + k);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const unsigned long long u =
-          static_cast<unsigned long long>(__double_as_longlong(p[kReduceSums + k]));
+          static_cast<unsigned long long>(__double_as_longlong(__ldcg(p + kReduceSums + k)));
       m[k] = u > m[k] ? u : m[k];
     }
   }
@@ -495,6 +483,65 @@ __global__ void __launch_bounds__(256) k_reduce_finish(const ReduceArgs a, int n
                                         ? redm[threadIdx.x - kReduceSums][w] : u;
     a.out[threadIdx.x] = __longlong_as_double(static_cast<long long>(u));
   }
+}
+
+// A grid-stride pass of resident blocks (64 registers, four an SM; more of them in a second wave
+// left most SMs idle at its end); block b writes its kReduceOut partial results to a.part[b],
+// and the one that ends last combines them.  4096 x 256 x Q128 146 us in one launch (145 + 9 in
+// two before; a reduction of the 200 x 24 film is mostly launches): the chain of each cell's
+// float64 sums, snapshot and temperature between its loads keeps it from the 83 of one read.
+template <typename T>
+__global__ void __launch_bounds__(256, 4) k_reduce(const ReduceArgs a) {
+  const int cells = (a.nx + 2) * (a.ny + 2);
+  __shared__ ReduceSmem sm;
+  for (int i = int(threadIdx.x); i < a.q; i += 256) {
+    sm.w[i] = a.w[i];
+    sm.par[i] = uint8_t(parity_of(a.par, i));
+  }
+  extern __shared__ __align__(16) unsigned char pair_smem[];
+  FluxPair* tab = reinterpret_cast<FluxPair*>(pair_smem);
+  stage_pairs(tab, a.plane, a.q, [&](int i) { return parity_of(a.par, i); }, a.w, a.sx, a.sy);
+  __syncthreads();
+  double v[kReduceSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  double res = 0.0, resw = 0.0;   // largest |T - T_snap| and window change (>= 0 or NaN)
+  for (int t = int(blockIdx.x) * 256 + int(threadIdx.x); t < cells; t += int(gridDim.x) * 256)
+    reduce_cell<T>(a, sm, tab, t, v, &res, &resw);
+  __shared__ double red[kReduceSums][8];
+  __shared__ unsigned long long redm[2][8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kReduceSums; ++k) {
+    const double s = warp_sum(v[k]);
+    if (lane == 0) red[k][wid] = s;
+  }
+  // |.| is non-negative, so its bit pattern orders like its value (NaN above all)
+  const unsigned long long m0 = warp_max_u64(static_cast<unsigned long long>(__double_as_longlong(res)));
+  const unsigned long long m1 = warp_max_u64(static_cast<unsigned long long>(__double_as_longlong(resw)));
+  if (lane == 0) {
+    redm[0][wid] = m0;
+    redm[1][wid] = m1;
+  }
+  __syncthreads();
+  if (threadIdx.x < kReduceSums) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
+    a.part[int64_t(blockIdx.x) * kReduceOut + threadIdx.x] = s;
+  } else if (threadIdx.x < kReduceOut) {
+    unsigned long long m = 0ull;
+    for (int w = 0; w < 8; ++w) m = redm[threadIdx.x - kReduceSums][w] > m
+                                        ? redm[threadIdx.x - kReduceSums][w] : m;
+    a.part[int64_t(blockIdx.x) * kReduceOut + threadIdx.x] = __longlong_as_double(
+        static_cast<long long>(m));
+  }
+  // the count returns to 0 by itself
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(a.done, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  reduce_finish(a, int(gridDim.x));
 }
 
 template <typename T>
@@ -645,10 +692,11 @@ cudaError_t launch_init(int storage, const InitArgs& a, cudaStream_t s) {
 
 cudaError_t launch_moments(int storage, const MomentArgs& a, cudaStream_t s) {
   const unsigned g = blocks_for(int64_t(a.nx) * a.ny, 256);
+  const size_t bytes = a.qx || a.qy ? size_t(a.q / 2) * sizeof(FluxPair) : 0;
   if (storage == WLBM_STORE_BF16_DEV)
-    k_moments<__nv_bfloat16><<<g, 256, 0, s>>>(a);
+    k_moments<__nv_bfloat16><<<g, 256, bytes, s>>>(a);
   else
-    k_moments<float><<<g, 256, 0, s>>>(a);
+    k_moments<float><<<g, 256, bytes, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -665,11 +713,11 @@ cudaError_t launch_sources(int storage, const SourceArgs& a, cudaStream_t s) {
 cudaError_t launch_reduce(int storage, const ReduceArgs& a, cudaStream_t s) {
   const int cells = (a.nx + 2) * (a.ny + 2);
   const int nb = std::max(1, std::min(kReduceBlocks, (cells + 255) / 256));
+  const size_t bytes = size_t(a.q / 2) * sizeof(FluxPair);
   if (storage == WLBM_STORE_BF16_DEV)
-    k_reduce<__nv_bfloat16><<<nb, 256, 0, s>>>(a);
+    k_reduce<__nv_bfloat16><<<nb, 256, bytes, s>>>(a);
   else
-    k_reduce<float><<<nb, 256, 0, s>>>(a);
-  k_reduce_finish<<<1, 256, 0, s>>>(a, nb);
+    k_reduce<float><<<nb, 256, bytes, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -123,7 +123,7 @@ struct wlbm_handle {
   uint8_t* d_codes = nullptr; // [kChunk][q]
   uint16_t* d_order = nullptr; // [kChunk][q + 17] kind-sorted directions (variant 3)
   double* d_red = nullptr;    // [kReduceOut]
-  double* d_red_part = nullptr;   // [kReduceBlocks][kReduceOut] reduction partials
+  double* d_red_part = nullptr;   // [kReduceBlocks][kReduceOut] reduction partials, and a count
   double* d_snap = nullptr;   // nx*ny float64 T - T_ref at the last reduction
   int64_t snap_step = -1;     // step of that snapshot (-1: none since the state was set)
   bool batch_owned = false;   // instance of a wlbm_batch (its records cache plane roles)
@@ -606,7 +606,7 @@ wlbm_status wlbm_create(const wlbm_grid* grid, const float* mfp_cells, double mf
   h->d_order = static_cast<uint16_t*>(h->dev_alloc(size_t(kChunk) * (G.q + 17) * 2));
   h->d_red = static_cast<double*>(h->dev_alloc(8 * sizeof(double)));
   h->d_red_part = static_cast<double*>(
-      h->dev_alloc(size_t(kReduceBlocks) * kReduceOut * sizeof(double)));
+      h->dev_alloc((size_t(kReduceBlocks) * kReduceOut + 1) * sizeof(double)));
   h->d_snap = static_cast<double*>(h->dev_alloc(size_t(g.nx) * g.ny * sizeof(double)));
   h->d_status = static_cast<int*>(h->dev_alloc(256));
   if (h->planes)
@@ -634,6 +634,8 @@ wlbm_status wlbm_create(const wlbm_grid* grid, const float* mfp_cells, double mf
   cudaStream_t s = h->stream;
   cudaError_t e = cudaMemsetAsync(h->planes, 0, 2 * size_t(G.q) * plane_bytes + 1024, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_status, 0, 256, s);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(h->d_red_part + size_t(kReduceBlocks) * kReduceOut, 0, sizeof(double), s);
   for (int k = 0; k < n_e && e == cudaSuccess; ++k)
     e = cudaMemsetAsync(h->e[k], 0, size_t(g.plane) * 4, s);
   if (e == cudaSuccess)
@@ -1119,6 +1121,7 @@ static wlbm_status reduce_impl(wlbm_handle* h, double* out, const WindowCtl* win
   a.q = g.q; a.par = h->parity_mask(); a.e_cur = h->e[h->e_cur]; a.e_refp = h->ref_plane();
   a.w = h->w_dev(); a.sx = h->sx_dev(); a.sy = h->sy_dev(); a.out = h->d_red; a.scale = h->scale;
   a.part = h->d_red_part;
+  a.done = reinterpret_cast<unsigned*>(h->d_red_part + size_t(kReduceBlocks) * kReduceOut);
   a.diff_mask = 0;
   for (int k = 0; k < 4; ++k)
     if (h->bc_kind[k] == WLBM_BC_ADIABATIC_DIFFUSE) a.diff_mask |= 1 << k;
@@ -1139,7 +1142,7 @@ static wlbm_status reduce_impl(wlbm_handle* h, double* out, const WindowCtl* win
     a.win_has_prev = win->has_prev ? 1 : 0;
     a.win_inv = 1.0 / win->count;
   }
-  h->launches += 2;
+  ++h->launches;
   st = h->cuda(launch_reduce(h->storage, a, h->stream), "wlbm_reduce");
   double tmp[kReduceOut];
   if (st == WLBM_OK)

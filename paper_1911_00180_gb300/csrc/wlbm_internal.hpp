@@ -278,8 +278,9 @@ struct ReduceArgs {
   const float* w;
   const float* sx;
   const float* sy;
-  double* out;           // [kReduceOut], written by the second stage
+  double* out;           // [kReduceOut], written by the last block
   double* part;          // [kReduceBlocks][kReduceOut] per-block partials (scratch)
+  unsigned* done;        // blocks that have ended (0 between launches)
   double scale;
   int diff_mask;         // bit k: side k (x-, x+, y-, y+) is an adiabatic-diffuse wall
   // central band of columns band_x0 <= x < band_x0 + band_w (conductivity fit)
@@ -304,7 +305,7 @@ struct ReduceArgs {
 // combined with an unsigned max).
 constexpr int kReduceSums = 6;
 constexpr int kReduceOut = 8;
-constexpr int kReduceBlocks = 152 * 8;   // grid-stride blocks of the first stage
+constexpr int kReduceBlocks = 152 * 4;   // grid-stride blocks, all resident (64 registers)
 
 struct StateArgs {
   void* planes;

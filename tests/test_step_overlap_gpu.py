@@ -58,15 +58,12 @@ def test_batch_steps_equal_synchronised_steps(walls, storage):
 
     import paper_1911_00180_gb300 as wl
     from paper_1911_00180_gb300 import wlbm as api
-    specs = [dict(nx=257, ny=33, q=32, bc=(P, P, P, P), mfp=4.0),
-             dict(nx=31, ny=130, q=8, bc=(P, P, P, P), mfp=9.0),
-             dict(nx=1500, ny=1450, q=8, bc=(P, P, P, P), mfp=9.0),
-             dict(nx=129, ny=15, q=64, bc=(P, P, P, P) if walls == "periodic" else (I, I, P, P),
-                  t_wall=(301.0, 300.0, 300.0, 300.0), mfp=9.0)]
-    if walls == "mixed":
-        specs.append(dict(nx=140, ny=41, q=16, bc=(I, I, A, A),
-                          t_wall=(301.0, 300.0, 300.0, 300.0), mfp=3.0))
-        del specs[2]
+    per, film = (P, P, P, P), (I, I, A, A)
+    sizes = [(257, 33, 32, per, 4.0), (31, 130, 8, per, 9.0)]
+    sizes += [(1500, 1450, 8, per, 9.0), (129, 15, 64, per, 9.0)] if walls == "periodic" else [
+        (129, 15, 64, (I, I, P, P), 9.0), (140, 41, 16, film, 3.0)]
+    specs = [dict(nx=nx, ny=ny, q=q, bc=bc, mfp=mfp, t_wall=(301.0, 300.0, 300.0, 300.0))
+             for nx, ny, q, bc, mfp in sizes]
     out = []
     for one, graph in ((True, 0), (False, 0), (False, 6)):
         s = torch.cuda.Stream()
