@@ -28,7 +28,8 @@ constexpr int kU = 8;                // directions in flight per thread (Q is a 
 
 // Where the direct kernels are the faster ones, in blocks the TMA form would have (152 SMs; up
 // to about one block an SM the TMA form leaves a ring's latency uncovered).  Microseconds a
-// step, TMA / direct: float32 256^2 x Q32 (38 tiles) 16.1 / 9.7, 300 x 400 x Q64 (87) 20.8 /
+// step, TMA / direct, both with ordinary launches (overlapping ones take 0.5-1.5 off either):
+// float32 256^2 x Q32 (38 tiles) 16.1 / 9.7, 300 x 400 x Q64 (87) 20.8 /
 // 14.5, 777 x 313 x Q40 (161) 22.9 / 18.0, 2048 x 128 x Q128 (160) 67.2 / 59.0, but 600^2 x Q64
 // (215) 37.9 / 39.7 and 640 x 700 x Q128 (250) 85.3 / 90.1; bfloat16 256^2 x Q32 17.9 / 12.0,
 // 400^2 x Q64 (116) 27.3 / 19.6, but 512^2 x Q64 (148) 23.2 / 28.2.  A backward pass with its
