@@ -25,6 +25,7 @@
 // lines run along the halo.
 #include <algorithm>
 
+#include "cluster_layout.hpp"
 #include "elem.cuh"
 #include "wlbm_internal.hpp"
 
@@ -32,46 +33,8 @@ namespace wlbm {
 
 namespace {
 
-constexpr int kClMax = 16;                 // blocks of a cluster (above 8: non-portable size)
 constexpr int kClMaxThreads = 1024;
-constexpr size_t kClSmem = 227 * 1024;
-constexpr int kClSums = 8;                 // partial sums of a wall's collected energy
 constexpr int kClFewThreads = 512;         // up to here a thread has 128 registers
-
-// Row length, in cells, of a block's arrays: its lines along the minor axis, halo included.  Odd,
-// so that lines next to one another start in different banks.
-__host__ __device__ inline int cl_line(int minor) { return (minor + 2) | 1; }
-
-// Shared memory of a block holding `lines` lines (halo included) of `line` cells.
-struct ClLayout {
-  uint32_t val, x, f, w, e, ep, tab, rho, part, src, total;
-  uint32_t plane;   // bytes of one direction's cells
-  uint32_t cells;
-};
-
-__host__ __device__ inline ClLayout cl_layout(int q, int lines, int line, int es) {
-  ClLayout L;
-  L.cells = uint32_t(lines) * uint32_t(line);
-  L.plane = (L.cells * uint32_t(es) + 15u) & ~15u;
-  uint32_t o = 0;
-  auto take = [&](uint32_t bytes) {
-    const uint32_t at = o;
-    o += (bytes + 15u) & ~15u;
-    return at;
-  };
-  L.val = take(2u * uint32_t(q) * L.plane);
-  L.x = take(2u * L.cells * 4u);                      // [2][cells] source terms
-  L.f = es == 2 ? take(2u * L.cells * 4u) : L.x;      // bfloat16: W E / scale
-  L.w = take(L.cells * 4u);                           // W_corr
-  L.e = take(L.cells * 4u);                           // local energy, own cells
-  L.ep = es == 2 ? take(L.cells * 4u) : L.e;          // and one step before
-  L.tab = take(2u * uint32_t(q) * 16u);
-  L.rho = take(3u * uint32_t(q) * 4u);                // re-emission fractions of y-, y+; w
-  L.src = take(uint32_t(q) * 4u);                     // plane of every direction
-  L.part = take(kClSums * 2u * uint32_t(lines > line ? lines : line) * 4u);
-  L.total = o;
-  return L;
-}
 
 __device__ __forceinline__ uint32_t cl_rank() {
   uint32_t r;
@@ -219,7 +182,7 @@ __global__ void __launch_bounds__(MAXT, 1)
   // offsets are those of the largest band, so that blocks can address one another's memory;
   // lines along the minor axis are contiguous, so that a halo is
   const int ws = cl_line(minor);
-  const ClLayout L = cl_layout(q, a.per + 2, ws, ES);
+  const ClLayout<uint32_t> L = cl_layout<uint32_t>(q, a.per + 2, ws, ES);
   const int sr = a.split_rows ? ws : 1, sc = a.split_rows ? 1 : ws;   // strides of rows, columns
   const int xb = (a.split_rows ? 0 : m0) - 1, yb = a.y_first + (a.split_rows ? m0 : 0) - 1;
   const bool mper = a.split_rows ? a.yper : a.xper;         // major axis periodic
@@ -518,7 +481,7 @@ const void* cluster_fn(int storage, int threads) {
 
 size_t cluster_bytes(const ClusterArgs& a, int es) {
   const int rows = a.y_last - a.y_first + 1;
-  return cl_layout(a.q, a.per + 2, cl_line(a.split_rows ? a.nx : rows), es).total;
+  return size_t(cl_bytes(a.q, a.per, a.split_rows ? a.nx : rows, es));
 }
 
 void cluster_config(int storage, const ClusterArgs& a, cudaStream_t s, cudaLaunchConfig_t* c,
@@ -561,7 +524,7 @@ bool cluster_plan(int storage, ClusterArgs* a) {
       c.split_rows = split;
       c.per = (major + nc - 1) / nc;
       c.nc = (major + c.per - 1) / c.per;   // no empty band
-      if (cluster_bytes(c, es) > kClSmem) continue;
+      if (!cl_fits(c.q, c.per, minor, es)) continue;
       const int64_t cells = int64_t(c.per) * minor;
       c.threads = int(std::min<int64_t>(kClMaxThreads, (std::max<int64_t>(cells, c.q) + 31) / 32 * 32));
       // cycles of a step: the directions of a thread's cells in turn, the halo, the barrier
