@@ -283,6 +283,8 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
  *                          only where an adiabatic-diffuse wall reads them: after a step
  *                          the ghost cells of periodic and isothermal sides hold what the
  *                          last boundary pass wrote (copies or wall values, not state).
+ *                          Steps run as one launch (below) leave the state's own copies and
+ *                          the wall values there.
  *                          Variant 3 never fuses the periodic mirrors: with
  *                          WLBM_OPT_FUSE_PERIODIC set it still runs the periodic pass.
  *                          A grid whose planes fit the shared memory of one thread-block
