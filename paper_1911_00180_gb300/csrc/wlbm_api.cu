@@ -1771,10 +1771,15 @@ struct wlbm_batch {
   std::vector<size_t> code_off, order_off;   // order_off in uint16 elements
   size_t code_bytes = 0, order_elems = 0;
   int total_tiles = 0, total_wall_blocks = 0;
-  std::vector<int> per;             // instances whose periodic edges need the separate pass
-  int2* d_per = nullptr;            // {instance, its first block column} of every block column
-  int per_cap = 0, per_blocks = 0, per_q = 0;   // of that pass; the largest Q among them
-  int64_t per_cells = 0;            // cells of those instances
+  // The separate periodic pass: {instance, its first block column} of every block column, written
+  // once.  Instances whose edges a fused step kernel mirrors itself come last, so that fusing or
+  // not, and the variant, only choose how many columns run.
+  struct PeriodicPass {
+    int blocks = 0, q = 0;   // block columns; the largest Q among the instances
+    int64_t cells = 0;       // their cells
+  };
+  int2* d_per = nullptr;
+  PeriodicPass per_all, per_unfused;
   // A captured chunk (the batched kernels read planes and phases at run time), two for the
   // replay parities, as for a single grid.
   TimedGraph graphs[2];
@@ -1850,36 +1855,38 @@ struct wlbm_batch {
       }
     return true;
   }
-  // Both axes periodic and fused: the step kernel mirrors the edges of that instance
-  // (not in variant 3, which has no mirror stores).
-  bool wraps(const wlbm_handle* x) const {
-    return fuse_periodic && variant != 3 && x->xper && x->yper && x->g.nx >= 2 && x->g.ny >= 2;
+  // Both axes periodic: a fused step kernel mirrors the edges of that instance (not in
+  // variant 3, which has no mirror stores).
+  bool fused() const { return fuse_periodic && variant != 3; }
+  bool can_wrap(const wlbm_handle* x) const {
+    return x->xper && x->yper && x->g.nx >= 2 && x->g.ny >= 2;
   }
-  // Instances of the periodic pass and its block table (false: it could not be uploaded).
-  bool classify() {
-    per.clear();
+  bool wraps(const wlbm_handle* x) const { return fused() && can_wrap(x); }
+  const PeriodicPass& per() const { return fused() ? per_unfused : per_all; }
+  // Instances of the periodic pass and its block table.
+  wlbm_status plan_periodic() {
     std::vector<int2> blocks;
-    per_q = 0;
-    per_cells = 0;
-    for (size_t k = 0; k < h.size(); ++k) {
-      const wlbm_handle* x = h[k];
-      if (!(x->xper || x->yper) || wraps(x)) continue;
-      per.push_back(int(k));
-      per_q = std::max(per_q, x->g.q);
-      per_cells += int64_t(x->g.nx) * x->g.ny;
-      const int first = int(blocks.size());
-      blocks.insert(blocks.end(), size_t(periodic_blocks(x->g.nx, x->g.ny, x->xper, x->yper)),
-                    make_int2(int(k), first));
+    PeriodicPass p;
+    for (const bool wrap : {false, true}) {
+      for (size_t k = 0; k < h.size(); ++k) {
+        const wlbm_handle* x = h[k];
+        if (!(x->xper || x->yper) || can_wrap(x) != wrap) continue;
+        p.q = std::max(p.q, x->g.q);
+        p.cells += int64_t(x->g.nx) * x->g.ny;
+        const int first = int(blocks.size());
+        blocks.insert(blocks.end(), size_t(periodic_blocks(x->g.nx, x->g.ny, x->xper, x->yper)),
+                      make_int2(int(k), first));
+      }
+      p.blocks = int(blocks.size());
+      (wrap ? per_all : per_unfused) = p;
     }
-    per_blocks = int(blocks.size());
-    if (per_blocks == 0) return true;
-    if (per_blocks > per_cap) {
-      d_per = static_cast<int2*>(dev_alloc(blocks.size() * sizeof(int2)));
-      per_cap = d_per ? per_blocks : 0;
-    }
-    return d_per && (!stream || cudaStreamSynchronize(stream) == cudaSuccess) &&
-           cudaMemcpy(d_per, blocks.data(), blocks.size() * sizeof(int2),
-                      cudaMemcpyHostToDevice) == cudaSuccess;
+    if (blocks.empty()) return WLBM_OK;
+    d_per = static_cast<int2*>(dev_alloc(blocks.size() * sizeof(int2)));
+    if (!d_per) return WLBM_ERR_OOM;
+    return (!stream || cudaStreamSynchronize(stream) == cudaSuccess) &&
+                   cudaMemcpy(d_per, blocks.data(), blocks.size() * sizeof(int2),
+                              cudaMemcpyHostToDevice) == cudaSuccess
+               ? WLBM_OK : WLBM_ERR_CUDA;
   }
   // Block and warp offsets of every instance in the batched grids.
   void layout() {
@@ -2033,7 +2040,9 @@ wlbm_status wlbm_batch_create(int32_t n, const wlbm_grid* grids, const float* co
   b->wide = b->all_tmap_w ? 1 : 0;
   std::memset(b->h_walls, 0, sizeof(BatchWalls) * n);
   b->layout();
-  if (!b->classify() || !b->tables_ok) {
+  const wlbm_status pst = b->plan_periodic();
+  if (pst == WLBM_ERR_OOM) return bad(pst, "wlbm_batch_create: device allocation failed");
+  if (pst != WLBM_OK || !b->tables_ok) {
     cudaGetLastError();
     return bad(WLBM_ERR_CUDA, "wlbm_batch_create: upload of the block tables failed");
   }
@@ -2095,9 +2104,9 @@ wlbm_status wlbm_batch_set_option(wlbm_batch* b, int32_t key, int64_t value) {
     b->variant = int(value);
     b->layout();
     b->drop_graph();
-    if (!b->classify() || !b->tables_ok) {
+    if (!b->tables_ok) {
       cudaGetLastError();
-      return b->fail(WLBM_ERR_CUDA, "wlbm_batch_set_option: upload of the block tables failed");
+      return b->fail(WLBM_ERR_CUDA, "wlbm_batch_set_option: upload of the tile tables failed");
     }
     return WLBM_OK;
   }
@@ -2134,10 +2143,6 @@ wlbm_status wlbm_batch_set_option(wlbm_batch* b, int32_t key, int64_t value) {
   if (key == WLBM_OPT_FUSE_PERIODIC && (value == 0 || value == 1)) {
     b->fuse_periodic = int(value);
     b->drop_graph();
-    if (!b->classify()) {
-      cudaGetLastError();
-      return b->fail(WLBM_ERR_CUDA, "wlbm_batch_set_option: upload of the block tables failed");
-    }
     return WLBM_OK;
   }
   if (key == WLBM_OPT_BF16_WIDE && (value == 0 || value == 1)) {
@@ -2230,9 +2235,11 @@ static wlbm_status batch_enqueue(wlbm_batch* b, int count, int every, TimedGraph
                    "wlbm_batch_step: walls");
       ++b->launches;
     }
-    if (st == WLBM_OK && b->per_blocks > 0) {
-      st = b->cuda(launch_periodic_batch(b->storage, b->d_inst, b->d_per, b->per_blocks, b->per_q,
-                                         b->per_cells <= kEarlyPeriodicCells, t, b->stream), "wlbm_batch_step: periodic");
+    const wlbm_batch::PeriodicPass& per = b->per();
+    if (st == WLBM_OK && per.blocks > 0) {
+      st = b->cuda(launch_periodic_batch(b->storage, b->d_inst, b->d_per, per.blocks, per.q,
+                                         per.cells <= kEarlyPeriodicCells, t, b->stream),
+                   "wlbm_batch_step: periodic");
       ++b->launches;
     }
     if (st != WLBM_OK) break;
