@@ -290,8 +290,9 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
  *                          A grid whose planes fit the shared memory of one thread-block
  *                          cluster (periodic or isothermal x sides; periodic, isothermal
  *                          or diffuse y sides of specularity 0; no sources; the other
- *                          options at their defaults) runs each chunk of steps as one
- *                          launch, with the same results bit for bit.
+ *                          options at their defaults) runs a chunk of steps, when they are
+ *                          enough to pay for it, as one launch, with the same results bit
+ *                          for bit.
  *   WLBM_OPT_GRAPH_STEPS   0 (default): launch every step's kernels directly; G > 0, a
  *                          multiple of 6: run chunks of G steps as one captured CUDA
  *                          graph (fewer launch gaps).  Replay needs a stream of its own:

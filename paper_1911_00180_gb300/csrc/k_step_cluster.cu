@@ -100,6 +100,12 @@ __device__ __forceinline__ int cl_mod(int v, int n) {
   return r < 0 ? r + n : r;
 }
 
+// Groups of threads that share the directions of `cells` cells, where a block has threads for
+// more than one: group g takes the eights g, g + groups, ...
+__device__ __forceinline__ int cl_groups(int cells, int q) {
+  return max(1, min(int(blockDim.x) / cells, q / 8));
+}
+
 // What a cell of the frame is.
 enum : int { kClVoid, kClIso, kClGhost, kClIn };   // outside, isothermal, diffuse ghost, interior
 
@@ -198,23 +204,37 @@ __device__ __noinline__ void cl_frame(const ClusterArgs& a, const unsigned char*
     if (BF && i == 0) a.e[o] = a.e_ref[o] = a.iso[side];
   }
   if (!a.xper && !a.yper) return;
-  for (int k = int(threadIdx.x); k < own * minor; k += int(blockDim.x)) {
-    const int M = k / minor, m = k - M * minor, at = (M + 1) * ws + m + 1;
+  const int cells = own * minor, groups = cl_groups(cells, q);
+  for (int k = int(threadIdx.x); k < cells * groups; k += int(blockDim.x)) {
+    const int group = k / cells, M = (k - group * cells) / minor, m = k - group * cells - M * minor;
+    const int at = (M + 1) * ws + m + 1;
     const int x = a.split_rows ? m : m0 + M, y = a.y_first + (a.split_rows ? m0 + M : m);
     const int right = a.xper && x == 0 ? a.nx : 0, left = a.xper && x == a.nx - 1 ? a.nx : 0;
     const int up = a.yper && y == 0 ? a.ny : 0, down = a.yper && y == a.ny - 1 ? a.ny : 0;
     if ((right | left | up | down) == 0) continue;
-    for (int j = 1; j < 9; ++j) {   // the images in x, in y and in both
-      const int jx = j % 3, jy = j / 3;
-      const int dx = jx == 0 ? 0 : jx == 1 ? right : -left, dy = jy == 0 ? 0 : jy == 1 ? up : -down;
-      if ((jx != 0 && dx == 0) || (jy != 0 && dy == 0)) continue;
-      const int64_t o = int64_t(y + dy + 2) * a.pitch + x + dx + kX0;
-#pragma unroll 8
-      for (int i = 0; i < q; ++i)
-        planes[int64_t(src[i]) * a.plane + o] = reinterpret_cast<const T*>(val + uint32_t(i) * plane)[at];
-      a.e[o] = E[at];
-      if (BF) a.e_ref[o] = Ep[at];
+    const int64_t o = int64_t(y + 2) * a.pitch + x + kX0;
+    auto images = [&](auto put) {   // in x, in y and in both
+      for (int j = 1; j < 9; ++j) {
+        const int jx = j % 3, jy = j / 3;
+        const int dx = jx == 0 ? 0 : jx == 1 ? right : -left;
+        const int dy = jy == 0 ? 0 : jy == 1 ? up : -down;
+        if ((jx == 0 || dx != 0) && (jy == 0 || dy != 0)) put(o + int64_t(dy) * a.pitch + dx);
+      }
+    };
+    for (int i = 8 * group; i < q; i += 8 * groups) {
+      T v[8];
+#pragma unroll
+      for (int d = 0; d < 8; ++d) v[d] = reinterpret_cast<const T*>(val + uint32_t(i + d) * plane)[at];
+      images([&](int64_t to) {
+#pragma unroll
+        for (int d = 0; d < 8; ++d) planes[int64_t(src[i + d]) * a.plane + to] = v[d];
+      });
     }
+    if (group != 0) continue;
+    images([&](int64_t to) {
+      a.e[to] = E[at];
+      if (BF) a.e_ref[to] = Ep[at];
+    });
   }
 }
 
@@ -265,44 +285,58 @@ __global__ void __launch_bounds__(MAXT, 1)
   __syncthreads();
 
   // ------------------------------------------------------------------- state read
-  for (int k = tid; k < (own + 2) * (minor + 2); k += nthr) {
-    const int M = k / (minor + 2), m = k - M * (minor + 2), at = M * ws + m;
-    const int r = a.split_rows ? M : m, c = a.split_rows ? m : M;
+  // Threads in turn along x, the axis that is contiguous in memory, whichever axis is split; a
+  // cell's directions eight at a time, all loaded before the first is stored (one load, one store
+  // left a latency per direction: one step of 11 x 11 x Q256 95 us, now 23).
+  const int rgroups = cl_groups(h * w, q);
+  for (int k = tid; k < h * w * rgroups; k += nthr) {
+    const int group = k / (h * w), r = (k - group * h * w) / w, c = k - (group * h + r) * w;
+    const int at = r * sr + c * sc;
     int x = xb + c, y = yb + r;
     float iso;
     const int kind = cl_kind(a, x, y, &iso);
     if (a.xper) x = cl_mod(x, a.nx);
     if (a.yper) y = cl_mod(y, a.ny);
     const int64_t o = int64_t(y + 2) * a.pitch + x + kX0;
-    float e = 0.f, wv = 0.f, ref = 0.f;
-    if (kind == kClIn || kind == kClGhost) {
-      e = a.e[o];
-      if (BF) ref = a.e_ref[o];
-      if (kind == kClIn) wv = a.wfield ? a.wfield[o] : a.w0;
-    } else if (kind == kClIso) {
-      ref = iso;   // an isothermal cell's values refer to the wall's own equilibrium
-    }
-    Wc[at] = wv;
-    Ec[at] = e;
-    if (BF) Ep[at] = ref;
-    const float fv = __fmul_rn(wv, e);
-    for (int b = 0; b < 2; ++b) {
-      if constexpr (BF) {
-        xbuf(b)[at] = __fmul_rn(fmaf(__fsub_rn(1.f, wv), ref, fv), a.inv_scale);
-        fbuf(b)[at] = __fmul_rn(fv, a.inv_scale);
-      } else {
-        xbuf(b)[at] = fv;
+    if (group == 0) {
+      float e = 0.f, wv = 0.f, ref = 0.f;
+      if (kind == kClIn || kind == kClGhost) {
+        e = a.e[o];
+        if (BF) ref = a.e_ref[o];
+        if (kind == kClIn) wv = a.wfield ? a.wfield[o] : a.w0;
+      } else if (kind == kClIso) {
+        ref = iso;   // an isothermal cell's values refer to the wall's own equilibrium
+      }
+      Wc[at] = wv;
+      Ec[at] = e;
+      if (BF) Ep[at] = ref;
+      const float fv = __fmul_rn(wv, e);
+      for (int b = 0; b < 2; ++b) {
+        if constexpr (BF) {
+          xbuf(b)[at] = __fmul_rn(fmaf(__fsub_rn(1.f, wv), ref, fv), a.inv_scale);
+          fbuf(b)[at] = __fmul_rn(fv, a.inv_scale);
+        } else {
+          xbuf(b)[at] = fv;
+        }
       }
     }
     const T* p = static_cast<const T*>(a.planes) + o;
     const bool held = kind == kClIn || kind == kClGhost;
-#pragma unroll 8
-    for (int i = 0; i < q; ++i) {
-      T v;
-      if (held) v = p[int64_t(src[i]) * a.plane];
-      else Elem<T>::st(&v, kind == kClIso && !BF ? __fmul_rn(wsm[i], iso) : 0.f);
-      reinterpret_cast<T*>(vbuf(0) + uint32_t(i) * L.plane)[at] = v;
-      reinterpret_cast<T*>(vbuf(1) + uint32_t(i) * L.plane)[at] = v;
+    for (int i = 8 * group; i < q; i += 8 * rgroups) {
+      T v[8];
+      if (held) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = p[int64_t(src[i + u]) * a.plane];
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          Elem<T>::st(&v[u], kind == kClIso && !BF ? __fmul_rn(wsm[i + u], iso) : 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        reinterpret_cast<T*>(vbuf(0) + uint32_t(i + u) * L.plane)[at] = v[u];
+        reinterpret_cast<T*>(vbuf(1) + uint32_t(i + u) * L.plane)[at] = v[u];
+      }
     }
   }
   auto put_table = [&](int t) {   // entries of step t from (i1, c1)
@@ -511,14 +545,21 @@ __global__ void __launch_bounds__(MAXT, 1)
     src[i] = (((code >> 4) & 1) ^ ((code & 8) ? 0 : 1)) * q + i;
   }
   __syncthreads();
-  for (int k = tid; k < cells; k += nthr) {
-    const int M = 1 + k / minor, m = 1 + k - (M - 1) * minor, at = M * ws + m;
-    const int64_t o = int64_t(yb + (a.split_rows ? M : m) + 2) * a.pitch + xb +
-                      (a.split_rows ? m : M) + kX0;
+  const int wgroups = cl_groups(cells, q);
+  for (int k = tid; k < cells * wgroups; k += nthr) {
+    const int group = k / cells, u = k - group * cells;
+    const int r = 1 + u / (w - 2), c = 1 + u - (r - 1) * (w - 2), at = r * sr + c * sc;
+    const int64_t o = int64_t(yb + r + 2) * a.pitch + xb + c + kX0;
     T* p = static_cast<T*>(a.planes) + o;
-#pragma unroll 8
-    for (int i = 0; i < q; ++i)
-      p[int64_t(src[i]) * a.plane] = reinterpret_cast<const T*>(vbuf(b) + uint32_t(i) * L.plane)[at];
+    for (int i = 8 * group; i < q; i += 8 * wgroups) {
+      T v[8];
+#pragma unroll
+      for (int d = 0; d < 8; ++d)
+        v[d] = reinterpret_cast<const T*>(vbuf(b) + uint32_t(i + d) * L.plane)[at];
+#pragma unroll
+      for (int d = 0; d < 8; ++d) p[int64_t(src[i + d]) * a.plane] = v[d];
+    }
+    if (group != 0) continue;
     a.e[o] = Ec[at];
     if (BF) a.e_ref[o] = Ep[at];
   }
@@ -567,6 +608,27 @@ cudaError_t configure_step_cluster() {
   return e;
 }
 
+// Steps a launch has to advance to pay for reading and writing the state through 16 SMs (0: none
+// do).  The other side is one-step launches (k_step_direct and the boundary passes).  Microseconds
+// of a call of n steps, calls in a row, cluster / one-step launches:
+//   a cell per thread: n = 1 33 / 21, n = 3 39 / 35, n = 4 44 / 46, n = 64 276 / 535 (64 x 64 x
+//     Q64); film 139 x 17 x Q32 20 / 20, 28 / 35, 33 / 46, 216 / 537; bfloat16 95 x 95 x Q64
+//     42 / 21, 56 / 47, 60 / 61, 474 / 783.
+//   few cells of 256 directions or more: n = 1 23 / 35, n = 64 437 / 1687 (film 11 x 11 x Q256).
+//   more cells per thread: n = 16 91 / 96, n = 32 158 / 183, n = 64 288 / 349 (134 x 134 x Q16);
+//     bfloat16 141 / 137, 238 / 267, 438 / 524 (1117 x 17 x Q32), 119 / 107, 201 / 198,
+//     371 / 391 (512 x 64 x Q16).  With fewer than eight directions to each of a thread's cells
+//     the one-step launches keep ahead: n = 64 394 / 342 (bfloat16 1878 x 29 x Q8), 426 / 390
+//     (1448 x 23 x Q16), 467 / 370 (float32 film 1512 x 24 x Q8), though 289 / 320 for float32
+//     189 x 189 x Q8.
+static int cluster_min_steps(const ClusterArgs& c) {
+  const int rows = c.y_last - c.y_first + 1;
+  const int64_t cells = int64_t(c.per) * (c.split_rows ? c.nx : rows);
+  const int64_t each = (cells + c.threads - 1) / c.threads;
+  if (each > 1) return 8 * each <= c.q ? 32 : 0;
+  return c.q >= 256 && cells * c.q <= 16384 ? 1 : 4;
+}
+
 bool cluster_plan(int storage, ClusterArgs* a) {
   const int es = storage == WLBM_STORE_BF16_DEV ? 2 : 4;
   const int rows = a->y_last - a->y_first + 1;
@@ -600,8 +662,9 @@ bool cluster_plan(int storage, ClusterArgs* a) {
       pick = c;
     }
   if (best == 0.0) return false;
+  pick.min_steps = cluster_min_steps(pick);
   *a = pick;
-  return true;
+  return pick.min_steps > 0;
 }
 
 cudaError_t launch_step_cluster(int storage, const ClusterArgs& a, cudaStream_t s) {

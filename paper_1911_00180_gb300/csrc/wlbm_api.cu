@@ -288,9 +288,10 @@ struct wlbm_handle {
       std::swap(e_cur, e_spare);
     }
   }
-  // The whole chunk in one launch: a small grid, the default step kernel, no sources.
-  bool cluster_on() const {
-    return cluster.nc > 0 && step_variant == 3 && ring_stages == 0 && tile_loop == 0 &&
+  // The whole chunk in one launch: a small grid, steps enough, the default step kernel, no
+  // sources.
+  bool cluster_on(int steps) const {
+    return cluster.nc > 0 && steps >= cluster.min_steps && step_variant == 3 && ring_stages == 0 && tile_loop == 0 &&
            n_src == 0 && !batch_owned && (!bf16() || bf16_wide);
   }
   void build_wall_segments();
@@ -768,7 +769,7 @@ static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every, TimedGrap
   auto selected = [&](int t) {
     return every > 0 && (cap ? t % every == 0 : h->prof_tick++ % every == 0);
   };
-  if (h->cluster_on()) {
+  if (h->cluster_on(count)) {
     int timed = 0;
     for (int t = 0; t < count; ++t) timed += selected(t);
     cudaEvent_t e0, e1;

@@ -108,8 +108,9 @@ struct ClusterArgs {
   float iso[4];           // e_eq(T_w) - e_ref of isothermal walls
   const float* rho;       // [8][q] re-emission fractions
   int y_first, y_last;    // computed cell rows (diffuse ghost rows included)
-  // set by cluster_plan: blocks, whether a block takes rows or columns, how many, threads
-  int nc, split_rows, per, threads;
+  // set by cluster_plan: blocks, whether a block takes rows or columns, how many, threads, the
+  // fewest steps of a launch
+  int nc, split_rows, per, threads, min_steps;
 };
 
 // Stable sort of one step's directions by kind = hop | paused << 3 (16 kinds): writes the
@@ -485,7 +486,8 @@ cudaError_t launch_adj_tma(const AdjArgs& a, const void* lam_map, const void* la
                            const void* tape_map, int tape_z0, const uint16_t* order,
                            int* status, cudaStream_t s);
 // Small grids: attributes, the bands of the cluster that holds the state (false when it does
-// not fit; fields up to y_last must be set but codes, order and steps) and the launch.
+// not fit or never pays; fields up to y_last must be set but codes, order and steps) and the
+// launch.
 cudaError_t configure_step_cluster();
 bool cluster_plan(int storage, ClusterArgs* a);
 cudaError_t launch_step_cluster(int storage, const ClusterArgs& a, cudaStream_t s);

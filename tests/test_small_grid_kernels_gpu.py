@@ -1,7 +1,7 @@
 """Which kernel the default options of a small grid take, by the names the profiler records, and
 the cluster launch where tests of equal bits had not reached it: more than 512 threads a block in
-float32, rows of diffuse ghost cells longer than a block, replayed graphs, and grids that change
-between cluster and one-step launches.  The one-step launches (WLBM_OPT_TILE_LOOP) give the
+float32, several cells a thread, replayed graphs, and grids that change between cluster and
+one-step launches; and the rule on steps and directions between the two.  The one-step launches (WLBM_OPT_TILE_LOOP) give the
 same bits."""
 import numpy as np
 import pytest
@@ -83,17 +83,29 @@ def test_direct_kernels_are_taken(kernels, nx, ny, q, bc, spec, speed, storage):
     h.close()
 
 
-@pytest.mark.parametrize("nx,ny,q,storage,walls", [
-    (128, 100, 8, 0, "periodic"), (128, 100, 8, 0, "film"), (200, 100, 8, 0, "duct"),
-    (200, 100, 8, 0, "channel"), (8176, 1, 8, 1, "tube"), (8176, 1, 8, 1, "film")])
-def test_large_blocks_equal_single_steps(kernels, nx, ny, q, storage, walls):
+@pytest.mark.parametrize("nx,ny,q,storage,walls,steps,kernel", [
+    (128, 100, 8, 0, "periodic", 11, "k_step_cluster<float, 1024"),
+    (128, 100, 8, 0, "film", 11, "k_step_cluster<float, 1024"),
+    (130, 130, 16, 0, "duct", 33, "k_step_cluster<float, 1024"),       # two cells per thread
+    (130, 130, 16, 0, "channel", 33, "k_step_cluster<float, 1024"),
+    (128, 128, 32, 1, "film", 32, "k_step_cluster<__nv_bfloat16, 1024"),
+    (1024, 16, 32, 1, "tube", 40, "k_step_cluster<__nv_bfloat16, 1024"),
+    (130, 130, 16, 0, "periodic", 31, "k_step_direct<float"),          # too few steps
+    (200, 100, 8, 0, "duct", 40, "k_step_direct<float"),               # too few directions
+    (8176, 1, 8, 1, "tube", 40, "k_step_direct<__nv_bfloat16"),
+    (40, 30, 24, 0, "film", 3, "k_step_direct<float"),
+    (40, 30, 24, 0, "film", 4, "k_step_cluster<float"),
+    (11, 11, 256, 0, "film", 1, "k_step_cluster<float"),
+    (128, 16, 256, 1, "periodic", 1, "k_step_direct<__nv_bfloat16")])
+def test_rule_and_equal_bits(kernels, nx, ny, q, storage, walls, steps, kernel):
     from paper_1911_00180_gb300 import wlbm as api
     bc, out = WALLS[walls], []
     for loop in (0, 1):
         h = _grid(nx, ny, q, bc, storage)
         h.wlbm_set_option(api.OPT_TILE_LOOP, loop)
-        names = kernels(lambda: h.wlbm_step(11))
-        assert loop or (len(names) == 1 and "k_step_cluster" in names[0] and "1024" in names[0]), names
+        names = [k for k in kernels(lambda: h.wlbm_step(steps)) if "k_step" in k]
+        assert loop or (len(names) == (1 if "cluster" in kernel else steps) and
+                        all(kernel in k for k in names)), names
         h.wlbm_step(2)
         out.append(_state(h, bc))
         h.close()
@@ -108,7 +120,7 @@ def test_graphs_and_changes_between_launches(kernels, walls, storage):
 
     from paper_1911_00180_gb300 import wlbm as api
     bc, out = WALLS[walls], []
-    for parts in (((12, 0, 41),), ((0, 0, 5), (0, 1, 4), (0, 0, 3), (12, 0, 12), (12, 1, 13), (0, 0, 4)),
+    for parts in (((12, 0, 41),), ((0, 0, 5), (0, 1, 3), (0, 0, 4), (12, 0, 12), (12, 1, 13), (0, 0, 4)),
                   ((0, 1, 41),)):
         s = torch.cuda.Stream()
         with torch.cuda.stream(s):
@@ -118,7 +130,8 @@ def test_graphs_and_changes_between_launches(kernels, walls, storage):
                 h.wlbm_set_option(api.OPT_TILE_LOOP, loop)
                 r0 = h.wlbm_get_option(api.OPT_GRAPH_REPLAYS)
                 names = kernels(lambda: h.wlbm_step(n))
-                assert all(("k_step_cluster" in k) == (loop == 0) for k in names if "k_step" in k), names
+                assert all(("k_step_cluster" in k) == (loop == 0 and n >= 4)
+                           for k in names if "k_step" in k and not graph), names
                 assert h.wlbm_get_option(api.OPT_GRAPH_REPLAYS) - r0 == (n // 12 if graph else 0)
             out.append(_state(h, bc))
             h.close()
