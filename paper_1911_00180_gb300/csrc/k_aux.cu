@@ -601,11 +601,11 @@ cudaError_t walls_t(const WallArgs& a, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t periodic_t(const PeriodicArgs& a, cudaStream_t s) {
+cudaError_t periodic_t(const PeriodicArgs& a, bool early, cudaStream_t s) {
   const int blocks = periodic_blocks(a.nx, a.ny, a.xper, a.yper);
   if (blocks == 0) return cudaSuccess;
   const dim3 grid(unsigned(blocks), a.q + (a.e_ref ? 2 : 1));
-  if (int64_t(a.nx) * a.ny <= kEarlyPeriodicCells)
+  if (early)
     launch_dependent(k_periodic<T>, grid, 256, 0, s, a);
   else
     k_periodic<T><<<grid, 256, 0, s>>>(a);
@@ -663,9 +663,9 @@ cudaError_t launch_walls(int storage, const WallArgs& a, cudaStream_t s) {
   return storage == WLBM_STORE_BF16_DEV ? walls_t<__nv_bfloat16>(a, s) : walls_t<float>(a, s);
 }
 
-cudaError_t launch_periodic(int storage, const PeriodicArgs& a, cudaStream_t s) {
-  return storage == WLBM_STORE_BF16_DEV ? periodic_t<__nv_bfloat16>(a, s)
-                                        : periodic_t<float>(a, s);
+cudaError_t launch_periodic(int storage, const PeriodicArgs& a, bool early, cudaStream_t s) {
+  return storage == WLBM_STORE_BF16_DEV ? periodic_t<__nv_bfloat16>(a, early, s)
+                                        : periodic_t<float>(a, early, s);
 }
 
 cudaError_t launch_range(const float* x, int64_t n, unsigned* out, cudaStream_t s) {

@@ -392,7 +392,7 @@ static wlbm_status refresh_periodic(wlbm_handle* h) {
   if (st != WLBM_OK) return st;
   pa.par = reinterpret_cast<const ParityMask*>(h->d_codes);
   ++h->launches;
-  return h->cuda(launch_periodic(h->storage, pa, h->stream), "periodic refresh");
+  return h->cuda(launch_periodic(h->storage, pa, false, h->stream), "periodic refresh");
 }
 
 // Diffuse re-emission fractions: tables 0-3 for the walls (inward normals +x, -x, +y,
@@ -797,6 +797,22 @@ static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every, TimedGrap
   wlbm_status st = WLBM_OK;
   for (int t = 0; t < count; ++t) {
     const uint8_t* codes = h->d_codes + size_t(t) * g.q;
+    StepArgs sa{};
+    sa.planes = h->planes; sa.plane = g.plane; sa.pitch = g.pitch; sa.rows = g.rows;
+    sa.nx = g.nx; sa.ny = g.ny; sa.q = g.q; sa.codes = codes; sa.w = h->w_dev();
+    sa.e_in = h->e[h->e_cur]; sa.e_out = h->e[h->e_spare]; sa.e_ref = h->ref_plane();
+    sa.wfield = h->field_w ? h->wfield : nullptr; sa.w0 = h->w0;
+    sa.scale = h->scale; sa.inv_scale = h->inv_scale;
+    sa.variant = h->step_variant; sa.status = h->d_status;
+    sa.xper = h->xper; sa.yper = h->yper; sa.wrap = wrap;
+    sa.tmap = h->has_tmap ? h->tmap : nullptr;
+    sa.ring_stages = h->ring_stages;
+    sa.loop_blocks = h->tile_loop ? h->loop_blocks : 0;
+    sa.wide = h->bf16_wide;
+    sa.tmap_w = h->has_tmap_w ? h->tmap_w : nullptr;
+    sa.order = h->d_order + size_t(t) * (g.q + 17);
+    int tiles_x = 0, tiles_y = 0;
+    tma_cover(h->bc_kind, g.nx, g.ny, &sa, &tiles_x, &tiles_y);
     if (any_wall) {
       WallArgs wa = h->walls;
       wa.codes = codes;
@@ -821,26 +837,18 @@ static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every, TimedGrap
       pa.ny = g.ny; pa.q = g.q; pa.codes = codes; pa.e_cur = h->e[h->e_cur];
       pa.e_ref = h->ref_plane();
       pa.xper = h->xper; pa.yper = h->yper;
-      st = h->cuda(launch_periodic(h->storage, pa, h->stream), "wlbm_step: periodic");
+      bool few = false;   // the step ahead ends soon after its first blocks do
+      if (h->step_variant == 3) {
+        int cbase_unused = 0;
+        if (h->bf16() && sa.wide) tma_cover_wide(sa, &cbase_unused, &tiles_x);
+        few = step_is_direct(h->storage, sa) || few_tiles(int64_t(tiles_x) * tiles_y, g.ny);
+      }
+      const bool early = periodic_early(int64_t(g.nx) * g.ny, cap != nullptr,
+                                        any_wall || h->n_src > 0, few);
+      st = h->cuda(launch_periodic(h->storage, pa, early, h->stream), "wlbm_step: periodic");
       if (st != WLBM_OK) return st;
       ++h->launches;
     }
-    StepArgs sa{};
-    sa.planes = h->planes; sa.plane = g.plane; sa.pitch = g.pitch; sa.rows = g.rows;
-    sa.nx = g.nx; sa.ny = g.ny; sa.q = g.q; sa.codes = codes; sa.w = h->w_dev();
-    sa.e_in = h->e[h->e_cur]; sa.e_out = h->e[h->e_spare]; sa.e_ref = h->ref_plane();
-    sa.wfield = h->field_w ? h->wfield : nullptr; sa.w0 = h->w0;
-    sa.scale = h->scale; sa.inv_scale = h->inv_scale;
-    sa.variant = h->step_variant; sa.status = h->d_status;
-    sa.xper = h->xper; sa.yper = h->yper; sa.wrap = wrap;
-    sa.tmap = h->has_tmap ? h->tmap : nullptr;
-    sa.ring_stages = h->ring_stages;
-    sa.loop_blocks = h->tile_loop ? h->loop_blocks : 0;
-    sa.wide = h->bf16_wide;
-    sa.tmap_w = h->has_tmap_w ? h->tmap_w : nullptr;
-    sa.order = h->d_order + size_t(t) * (g.q + 17);
-    int tx_unused = 0, ty_unused = 0;
-    tma_cover(h->bc_kind, g.nx, g.ny, &sa, &tx_unused, &ty_unused);
     cudaEvent_t e0, e1;
     st = timing(selected(t) ? 1 : 0, 1, &e0, &e1);
     if (st == WLBM_OK && e0)
@@ -1647,7 +1655,9 @@ wlbm_status wlbm_adjoint_backward(wlbm_handle* h, const float* dJ_dT, const floa
         pa.planes = slot; pa.plane = g.plane; pa.pitch = g.pitch; pa.nx = g.nx; pa.ny = g.ny;
         pa.q = g.q; pa.codes = codes; pa.e_cur = A.erec[ec]; pa.e_ref = nullptr;
         pa.xper = h->xper; pa.yper = h->yper; pa.tape = 1;
-        ok(launch_periodic(h->storage, pa, s), "adjoint: periodic");
+        ok(launch_periodic(h->storage, pa,
+                           periodic_early(int64_t(g.nx) * g.ny, false, false, false), s),
+           "adjoint: periodic");
       }
       if (j + 1 < kc) {
         StepArgs sa{};

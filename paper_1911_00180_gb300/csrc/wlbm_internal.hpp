@@ -219,11 +219,24 @@ __host__ __device__ inline int wall_chunk_segment(int nseg, const WallSeg* seg, 
 #endif
 
 
-// Periodic passes of up to this many cells start as dependents of the step ahead of them; on
-// larger grids their waiting blocks cost the step's last waves more than the early start gives
-// (early / not, us a step: 512^2 x Q64 27.1 / 27.9, 1024^2 x Q64 99.9 / 100.4, 1400^2 x Q32
-// 89.4 / 89.5, 2048^2 x Q16 99.1 / 98.4, 2048^2 x Q64 341.2 / 338.6, bfloat16 194.5 / 191.8).
+// Which periodic passes start as dependents of the kernel ahead of them.  What that gives is the
+// host's launch gap and the pass' own start; what it costs, behind a step of tiles, is the step's
+// last waves, where the waiting blocks sit.  Early / not, us a step:
+//   launched one by one, up to this many cells: 512^2 x Q64 27.1 / 27.9, 1024^2 x Q64 96.4 / 98.1,
+//     2048 x 1024 x Q64 177.1 / 178.0; above: 2048^2 x Q16 99.1 / 98.4, 2048^2 x Q64 341.2 / 338.6,
+//     bfloat16 194.5 / 191.8.
+//   in a graph, which has no such gaps, behind a step of many tiles: 1024^2 x Q8 17.3 / 16.7,
+//     1500 x 1000 x Q64 132.1 / 130.0, bfloat16 87.3 / 84.0, 700^2 x Q32 (300 tiles) 25.1 / 24.8;
+//     of fewer, 3000 x 100 x Q24 (192) 14.1 / 14.7, bfloat16 700^2 x Q32 (150) 17.9 / 18.5, but not
+//     where the pass is mostly columns, a sector for each of their cells: 129 x 1800 x Q48 (258)
+//     28.8 / 27.6, bfloat16 (129) 24.9 / 24.2.
+//   in a graph behind another boundary pass (1024^2 x Q8 with walls 17.3 / 17.7) or a step of the
+//     direct kernel (512^2 x Q64 26.5 / 27.1, 256^2 x Q32 7.0 / 7.6).
 constexpr int64_t kEarlyPeriodicCells = int64_t(1) << 21;
+inline bool few_tiles(int64_t tiles, int ny) { return tiles <= 200 && ny <= 1024; }
+inline bool periodic_early(int64_t cells, bool graph, bool after_pass, bool few) {
+  return cells <= kEarlyPeriodicCells && (!graph || after_pass || few);
+}
 
 struct PeriodicArgs {
   void* planes;
@@ -506,7 +519,8 @@ bool batch_persistent_stages_ok(int storage, int stages);
 cudaError_t launch_batch_persistent(int storage, int stages, const PersistArgs& p, int max_q,
                                     int grid, bool any_spec, cudaStream_t s);
 cudaError_t launch_walls(int storage, const WallArgs& a, cudaStream_t s);
-cudaError_t launch_periodic(int storage, const PeriodicArgs& a, cudaStream_t s);
+// (early: as a programmatic dependent, see periodic_early)
+cudaError_t launch_periodic(int storage, const PeriodicArgs& a, bool early, cudaStream_t s);
 // Blocks per plane of a grid's periodic pass, and the pass of step t of every instance of a batch
 // that needs one: total_blocks block columns, blocks[b] = {instance, its first column}; max_q
 // the largest Q among them.
