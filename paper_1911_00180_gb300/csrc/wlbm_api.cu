@@ -150,6 +150,8 @@ struct wlbm_handle {
   int tile_loop = 0;          // variant 3: 1 = resident blocks loop over the tiles
   int loop_blocks = 0;        // blocks of that grid (set with the options)
   int fuse_periodic = 0;      // 1: both axes periodic, the step kernel mirrors the edges
+  bool images = false;        // the ghost cells behind periodic links are the state's copies
+                              // (steps with mirrors read and keep them; others write them first)
   // per energy-plane role and replay parity (consecutive replays alternate, so a graph's
   // event pairs are read while the other one runs)
   TimedGraph graphs[3][2];
@@ -288,6 +290,13 @@ struct wlbm_handle {
       std::swap(e_cur, e_spare);
     }
   }
+  // Both axes periodic and fused: the step kernel mirrors the edges itself (grids of 2+ cells;
+  // variant 3 has no mirror stores, and sources must reach the ghost copies through the
+  // periodic pass).
+  bool wraps() const {
+    return fuse_periodic && step_variant != 3 && xper && yper && g.nx >= 2 && g.ny >= 2 &&
+           n_src == 0;
+  }
   // The whole chunk in one launch: a small grid, steps enough, the default step kernel, no
   // sources.
   bool cluster_on(int steps) const {
@@ -392,6 +401,7 @@ static wlbm_status refresh_periodic(wlbm_handle* h) {
   if (st != WLBM_OK) return st;
   pa.par = reinterpret_cast<const ParityMask*>(h->d_codes);
   ++h->launches;
+  h->images = true;
   return h->cuda(launch_periodic(h->storage, pa, false, h->stream), "periodic refresh");
 }
 
@@ -788,11 +798,7 @@ static wlbm_status enqueue_steps(wlbm_handle* h, int count, int every, TimedGrap
     return st;
   }
   const bool any_wall = h->walls.nseg > 0;
-  // both axes periodic: the step kernel mirrors the edges itself (grids of 2+ cells)
-  // (variant 3 has no mirror stores: there the separate periodic pass runs)
-  // (sources must reach the ghost copies through the periodic pass: no mirrors with them)
-  const bool wrap = h->fuse_periodic && h->step_variant != 3 && h->xper && h->yper &&
-                    g.nx >= 2 && g.ny >= 2 && h->n_src == 0;
+  const bool wrap = h->wraps();
   const bool any_per = (h->xper || h->yper) && !wrap;
   wlbm_status st = WLBM_OK;
   for (int t = 0; t < count; ++t) {
@@ -923,6 +929,15 @@ wlbm_status wlbm_step(wlbm_handle* h, int64_t n) {
   if (n < 0) return h->fail(WLBM_ERR_INVALID_ARG, "wlbm_step: negative step count");
   const Geom& g = h->g;
   const bool graphs = h->graph_steps > 0 && h->stream != nullptr;
+  if (n > 0) {
+    // mirrors are copies of the step before: after steps without them, or a checkpoint of such
+    // steps, the first one needs them made
+    if (h->wraps() && !h->images) {
+      const wlbm_status st = refresh_periodic(h);
+      if (st != WLBM_OK) return st;
+    }
+    h->images = h->wraps();
+  }
   while (n > 0) {
     const int ch = int(std::min<int64_t>(n, graphs ? h->graph_steps : kChunk));
     const int slot = h->slot;
@@ -1436,6 +1451,7 @@ wlbm_status wlbm_load(wlbm_handle* h, const void* src, size_t size) {
   h->build_wall_segments();
   h->drop_graphs();
   h->snap_step = -1;
+  h->images = false;
   h->adj.ready = false;
   const unsigned char* p = in + ckpt_cursor_bytes(g.q);
   unsigned char* planes = static_cast<unsigned char*>(h->planes);
@@ -2301,6 +2317,14 @@ wlbm_status wlbm_batch_step(wlbm_batch* b, int64_t n) {
   if (n < 0) return b->fail(WLBM_ERR_INVALID_ARG, "wlbm_batch_step: negative step count");
   const int ni = int(b->h.size());
   const bool graphs = b->graph_steps > 0 && b->stream;
+  for (int k = 0; k < ni && n > 0; ++k) {   // mirrors: as in wlbm_step
+    wlbm_handle* x = b->h[k];
+    if (b->wraps(x) && !x->images) {
+      const wlbm_status st = refresh_periodic(x);
+      if (st != WLBM_OK) return b->fail(st, "instance " + std::to_string(k) + ": " + x->err);
+    }
+    x->images = b->wraps(x);
+  }
   while (n > 0) {
     const int ch = int(std::min<int64_t>(n, graphs ? b->graph_steps : kBatchChunk));
     wlbm_status st = b->cuda(cudaEventSynchronize(b->ev), "wlbm_batch_step");
