@@ -359,7 +359,8 @@ __global__ void k_adj_seed(const AdjArgs a, const float* dJ_dT, const float* dJ_
 }
 
 // dW_corr/dMFP (Eq. W-correction with W = v/MFP: a function of m = MFP/v, so dW_corr/dMFP =
-// (dW_corr/dm) / v).  Rounded operation by operation: a fused one would give other bits.
+// (dW_corr/dm) / v).  Rounded operation by operation, as the host rounds them; the exponential
+// of relax_mode 1 is the device's, which may differ from the host's in its last bit (float64).
 __device__ __forceinline__ float dw_dmfp(const AdjMfp& a, int cell) {
   const double m = __ddiv_rn(a.mfp ? double(a.mfp[cell]) : a.uniform, a.speed);
   if (isinf(m)) return 0.f;

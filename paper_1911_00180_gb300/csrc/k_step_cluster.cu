@@ -17,9 +17,11 @@
 //   * Diffuse walls (horizontal, specularity 0) collect and re-emit in shared memory between
 //     two steps, with the sums in the wall pass's order.
 // What bounds it: the latency of Q updates per cell with one block of threads an SM, the halo
-// and the barrier; not bandwidth.  Cycles of a step on 16 blocks, 64 x 64 x Q16: update 1250,
-// table 260, halo 960, barrier 1000 (1.8 us a step, 14.5 with launches); the 200 x 24 x Q32
-// film: 4050, 240, walls 1650, halo 920, barrier 1480 (3.9 us, 22).  Halos filled by an
+// and the barrier; not bandwidth.  Cycles of a step on 16 blocks at 2.07 GHz, 64 x 64 x Q16:
+// update 1340, table 260, halo 990, barrier 950, 3700 in all (1.8 us a step, 14.5 with
+// launches); the 200 x 24 x Q32 film: 4140, 240, walls 1690, halo 880, barrier 1350, 8400 in all
+// (4.0 us, 22 with launches).  A launch adds 10-20 us, with few directions half of it the state's
+// reads and writes (cluster_min_steps has the rule that follows).  Halos filled by an
 // element loop over (direction, cell) took 4900 cycles (the index divisions), halos across
 // rows of the other axis 3100 (scattered remote stores), so a thread keeps its halo cell and
 // lines run along the halo.
